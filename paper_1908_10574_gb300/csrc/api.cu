@@ -162,6 +162,26 @@ int prepare_seqs(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int32_t
     return CM_OK;
 }
 
+namespace {
+
+// rows of the longest of the n streams that subjects [s0, s1) split into (at the subject
+// boundaries nearest to equal shares, as the kernels split them)
+int64_t longest_stream(const int64_t* srow, int32_t s0, int32_t s1, int n)
+{
+    int64_t longest = 0;
+    int32_t prev = s0;
+    for (int i = 1; i <= n; ++i) {
+        const int64_t key = srow[s0] + (srow[s1] - srow[s0]) * i / n;
+        int32_t s = (int32_t)(std::lower_bound(srow + prev, srow + s1, key) - srow);
+        if (s > prev && key - srow[s - 1] < srow[s] - key) --s;
+        longest = std::max(longest, srow[s] - srow[prev]);
+        prev = s;
+    }
+    return longest;
+}
+
+}  // namespace
+
 // ---- execution --------------------------------------------------------------------------
 int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64_t* d_omap,
              uint32_t flags)
@@ -184,7 +204,6 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     ENSURE(B_STREAM, nrows_total + 64, d_stream);
     int r;
     if ((r = copy_in(c, d_blocks, plan.blocks.data(), plan.blocks.size() * sizeof(SwBlock), false))) return r;
-    if ((r = copy_in(c, d_tasks, plan.tasks.data(), plan.tasks.size() * sizeof(SwTask), false))) return r;
     if ((r = copy_in(c, d_ids, plan.ids.data(), plan.ids.size() * sizeof(int32_t), false))) return r;
     if (!plan.dev_lists)
         if ((r = copy_in(c, d_srow, plan.srow.data(), plan.srow.size() * sizeof(int64_t), false))) return r;
@@ -212,54 +231,155 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     a.beta = P.beta;
     a.sat_thr = (flags & CM_FORCE_INT32) ? -1 : P.sat_thr;   // -1: every pair goes to int32
 
-    // boundary buffer for multi-pass queries and for the int32 rerun
-    // even, so the pair-mode records (16 bytes per two rows) stay 16-byte aligned
+    // Launches.  All single-query tasks run in one launch, each CTA a contiguous range of them
+    // of an equal share of the cost: first the tasks of several passes, then tile by tile (the
+    // plan's order).  The query pairs run in one persistent launch per (register tile, mode)
+    // bin.  (Builds without the single-query launcher give its tasks a launch per bin too.)
+    struct Launch {
+        int R, mode, grid, warps_per_cta;
+        size_t i0, i1;
+        bool single;
+        int64_t warps;                  // boundary slots (0: no task has a second pass)
+    };
+    std::vector<Launch> launches;
+    size_t n_single = 0;
+    std::vector<SwUnit> units;
+    int32_t *d_ranges = nullptr, *d_tickets = nullptr;
+    SwUnit* d_units = nullptr;
+    int64_t piped_rows = 0;
+    if (launch_sw16_single) {
+        std::vector<size_t> idx;
+        auto single = [&](const SwTask& t) { return t.mode == kModeTwo || t.mode == kModeTwo16; };
+        for (size_t i = 0; i < plan.tasks.size(); ++i)
+            if (single(plan.tasks[i])) idx.push_back(i);
+        n_single = idx.size();
+        if (n_single > 0) {
+            std::stable_partition(idx.begin(), idx.end(),
+                                  [&](size_t x) { return plan.tasks[x].npass > 1; });
+            std::vector<double> cost;
+            double total = 0;
+            for (size_t i : idx) {
+                const SwTask& t = plan.tasks[i];
+                SwUnit u{t.block, t.k, t.s0, t.s1, t.npass, 0, t.npass, t.mode, t.R, 0, -1};
+                const bool two16 = t.mode == kModeTwo16;
+                int64_t rows = INT32_MAX;
+                double steps = (double)plan.keys[i].first / ((double)t.R * t.npass);
+                if (!plan.dev_lists) {
+                    const int64_t* srow = plan.srow.data() + plan.blocks[t.block].srow;
+                    rows = srow[t.s1] - srow[t.s0];
+                    steps = (double)longest_stream(srow, t.s0, t.s1, two16 ? 4 : 2);
+                }
+                steps += kRowGroup * (two16 ? 16 : 32);       // filling the wavefront
+                const bool piped = t.npass > 1 && piped_rows + rows <= kPipedRows;
+                if (piped) {
+                    u.rows = (int32_t)rows;
+                    u.bnd_row = piped_rows;
+                    piped_rows += rows;
+                }
+                const int n = piped ? t.npass : 1;
+                for (int p = 0; p < n; ++p) {
+                    if (piped) { u.pass = p; u.pass_end = p + 1; }
+                    units.push_back(u);
+                    cost.push_back(steps * t.R * (t.npass / n));
+                    total += cost.back();
+                }
+            }
+            const int64_t nu = (int64_t)units.size();
+            if (nu >= INT32_MAX) return fail(c, CM_ERR_ARG, "too many tasks");
+            const int grid = (int)std::min<int64_t>(nu, c->num_sms);
+            std::vector<int32_t> ranges(1, 0);
+            double sum = 0;
+            for (int64_t t = 0; t < nu; ++t) {
+                // CTA b ends at the first unit that reaches its share, leaving one for the others
+                sum += cost[t];
+                const int64_t b = (int64_t)ranges.size();
+                if (b < grid && (sum * grid >= total * b || nu - t - 1 == grid - b))
+                    ranges.push_back((int32_t)t + 1);
+            }
+            ranges.push_back((int32_t)nu);
+            ENSURE(B_UNITS, nu, d_units);
+            ENSURE(B_RANGE, 2 * grid + 1 + nu, d_ranges);
+            d_tickets = d_ranges + grid + 1;
+            if ((r = copy_in(c, d_units, units.data(), units.size() * sizeof(SwUnit), false))) return r;
+            if ((r = copy_in(c, d_ranges, ranges.data(), ranges.size() * sizeof(int32_t), false))) return r;
+            CUDA_TRY(cudaMemsetAsync(d_tickets, 0, (grid + nu) * sizeof(int32_t), st));
+            const int warps = (int)std::min<int64_t>(kSingleWarps, (nu + grid - 1) / grid);
+            launches.push_back({0, kModeTwo, grid, warps, 0, n_single, true, 0});
+            // the plan's remaining tasks, in its order
+            std::vector<SwTask> t2;
+            std::vector<int> r2;
+            for (size_t i = 0; i < plan.tasks.size(); ++i)
+                if (!single(plan.tasks[i])) {
+                    t2.push_back(plan.tasks[i]);
+                    r2.push_back(plan.task_R[i]);
+                }
+            plan.tasks.swap(t2);
+            plan.task_R.swap(r2);
+        }
+    }
+    for (size_t i0 = 0; i0 < plan.tasks.size();) {
+        const int key = plan.task_R[i0];
+        size_t i1 = i0;
+        while (i1 < plan.tasks.size() && plan.task_R[i1] == key) ++i1;
+        const int64_t resident = (int64_t)c->num_sms * sw16_occupancy(c, key / 4, W, key % 4);
+        launches.push_back({key / 4, key % 4, (int)std::min<int64_t>((int64_t)(i1 - i0), resident), W,
+                            i0, i1, false, 0});
+        i0 = i1;
+    }
+    if ((int)launches.size() > kTaskBins)
+        return fail(c, CM_ERR_INTERNAL, "more launch bins than task tickets");
+    if ((r = copy_in(c, d_tasks, plan.tasks.data(), plan.tasks.size() * sizeof(SwTask), false))) return r;
+
+    // boundary buffer of the tasks with several column passes (a slot per resident warp; even
+    // strides, so the records of two rows stay 16-byte aligned).  Launches alternate between
+    // two streams and launches of one stream share its slots.
     const int64_t stride = (std::max<int64_t>(plan.max_warp_rows, P.maxlen) + 64 + 1) & ~(int64_t)1;
-    int max_ctas = 0;
-    for (int R = 1; R <= 32; ++R)
-        for (int mode = 0; mode < 4; ++mode)
-            max_ctas = std::max(max_ctas, c->num_sms * sw16_occupancy(c, R, W, mode));
-    const int64_t nwarps = std::max<int64_t>(std::max<int64_t>((int64_t)max_ctas * W,
-                                             (int64_t)c->num_sms * std::max(1, sw32_ctas_per_sm())),
-                                             (int64_t)c->num_sms * kLongSlots);
+    int64_t slots[2] = {0, 0};
+    for (size_t l = 0; l < launches.size(); ++l) {
+        Launch& L = launches[l];
+        bool passes = false;
+        if (L.single) {
+            for (const SwUnit& u : units) passes = passes || u.pass_end - u.pass > 1;
+        } else {
+            for (size_t i = L.i0; i < L.i1 && !passes; ++i) passes = plan.tasks[i].npass > 1;
+        }
+        L.warps = passes ? (int64_t)L.grid * L.warps_per_cta : 0;
+        slots[(l + 1) & 1] = std::max(slots[(l + 1) & 1], L.warps);
+    }
     uint2* d_bnd;
-    ENSURE(B_BND, 2 * nwarps * stride, d_bnd);     // one half per stream
+    piped_rows = (piped_rows + 1) & ~(int64_t)1;
+    ENSURE(B_BND, (slots[0] + slots[1]) * stride + piped_rows, d_bnd);
     a.bnd_stride = stride;
 
-    // One persistent launch per (register tile, mode) bin, longest tasks first within it.
-    // Consecutive bins alternate between the context stream and the auxiliary stream, so the
-    // next bin's CTAs take the SMs that the previous bin's CTAs leave as its queue drains
-    // (launch tails overlap); each stream has its own half of the boundary buffer.
+    // Consecutive launches alternate between the context stream and the auxiliary stream, so
+    // the next one's CTAs take the SMs that the previous one's leave as its queue drains
+    // (launch tails overlap).
     CUDA_TRY(cudaEventRecord(c->ev[0], st));
     CUDA_TRY(cudaEventRecord(c->fork, st));
     CUDA_TRY(cudaStreamWaitEvent(c->aux, c->fork, 0));
-    size_t i0 = 0;
-    int bin = 0;
     cudaError_t le = cudaSuccess;
-    while (i0 < plan.tasks.size() && le == cudaSuccess && bin < kTaskBins) {
-        const int key = plan.task_R[i0];
-        const int R = key / 4, mode = key % 4;
-        size_t i1 = i0;
-        while (i1 < plan.tasks.size() && plan.task_R[i1] == key) ++i1;
-        a.tasks = d_tasks + i0;
-        a.ntasks = (int32_t)(i1 - i0);
-        a.task_counter = d_flags + 8 + bin;
-        const int occ = sw16_occupancy(c, R, W, mode);
-        const int grid = (int)std::min<int64_t>(a.ntasks, (int64_t)c->num_sms * occ);
-        a.bnd = d_bnd + (bin & 1) * nwarps * stride;
-        le = launch_sw16(R, W, mode, grid, a, (bin & 1) ? c->aux : st);
+    for (size_t l = 0; l < launches.size() && le == cudaSuccess; ++l) {
+        const Launch& L = launches[l];
+        const int side = (int)(l + 1) & 1;
+        a.tasks = d_tasks + L.i0;
+        a.ntasks = (int32_t)(L.i1 - L.i0);
+        a.task_counter = L.single ? d_tickets : d_flags + 8 + l;
+        a.bnd = d_bnd + piped_rows + (side ? slots[0] : 0) * stride;
+        a.units = d_units;
+        a.ranges = d_ranges;
+        a.progress = L.single ? d_tickets + L.grid : nullptr;
+        a.piped = d_bnd;
+        const cudaStream_t ls = side ? c->aux : st;
+        le = L.single ? launch_sw16_single(L.grid, L.warps_per_cta, a, ls)
+                      : launch_sw16(L.R, W, L.mode, L.grid, a, ls);
         c->stats.launches += 1;
         c->stats.sw16_launches += 1;
-        i0 = i1;
-        ++bin;
     }
     // join the auxiliary stream before any return, so no launch of this call outlives it
     CUDA_TRY(cudaEventRecord(c->join, c->aux));
     CUDA_TRY(cudaStreamWaitEvent(st, c->join, 0));
     CUDA_TRY(le);
-    if (i0 < plan.tasks.size()) return fail(c, CM_ERR_INTERNAL, "more launch bins than task tickets");
     CUDA_TRY(cudaEventRecord(c->ev[1], st));
-    a.bnd = d_bnd;
 
     // int32 rescoring of every pair the int16 pass marked as possibly saturated
     PairRef* d_pref;
@@ -292,14 +412,17 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         if ((r = copy_in(c, d_pref, lst.data(), lst.size() * sizeof(PairRef), false))) return r;
         int32_t nlong = 0;
         while (nlong < n && is_long(lst[nlong])) ++nlong;
+        if (c->sw32_occ == 0) c->sw32_occ = std::max(1, sw32_ctas_per_sm());
+        const int64_t grid32 = std::min<int64_t>(n - nlong, (int64_t)c->num_sms * c->sw32_occ);
+        const int64_t grid_long = std::min<int64_t>(nlong, c->num_sms);
+        ENSURE(B_BND, std::max(grid32, grid_long * kLongSlots) * stride, d_bnd);
+        a.bnd = d_bnd;
         if (nlong > 0) {
-            CUDA_TRY(launch_long_sw32((int)std::min<int64_t>(nlong, c->num_sms), a, d_pref, nlong,
-                                      d_flags + 5, st));
+            CUDA_TRY(launch_long_sw32((int)grid_long, a, d_pref, nlong, d_flags + 5, st));
             c->stats.launches += 1;
         }
         if (n > nlong) {
-            const int grid = (int)std::min<int64_t>(n - nlong, (int64_t)c->num_sms * std::max(1, sw32_ctas_per_sm()));
-            CUDA_TRY(launch_sw32(16, grid, a, d_pref + nlong, n - nlong, d_flags + 3, st));
+            CUDA_TRY(launch_sw32(16, (int)grid32, a, d_pref + nlong, n - nlong, d_flags + 3, st));
             c->stats.launches += 1;
         }
         // every full round rescored `cap` distinct slots (a rescored slot no longer holds the
@@ -331,7 +454,26 @@ int64_t plan_blocks(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& id
     int64_t slots = 0;
     std::vector<int32_t> a_ids, b_ids;
     plan.srow.push_back(0);
-    const int64_t target = (int64_t)c->W * c->rows_per_warp;
+    // the queries of a block, two by two: fn(k, hi, subjects of k, subjects of the last one)
+    auto each_query = [&](const BlockReq& r, auto&& fn) {
+        for (int64_t k = 0; k < r.a_count; k += 2) {
+            const bool hi = k + 1 < r.a_count;
+            const int32_t ns_lo = (r.kind == kTri) ? (int32_t)k : (int32_t)r.b_count;
+            const int32_t ns = (r.kind == kTri) ? (int32_t)(hi ? k + 1 : k) : (int32_t)r.b_count;
+            fn(k, hi, ns_lo, ns);
+        }
+    };
+    TaskSizer sizer(c->W, c->num_sms, c->rows_per_warp);
+    std::vector<int64_t> pre;                        // rows of the subjects before s
+    for (const BlockReq& r : req) {
+        pre.assign(1, 0);
+        for (int64_t s = 0; s < r.b_count; ++s)
+            pre.push_back(pre.back() + stream_rows(P.len(ids[r.b_begin + s])));
+        each_query(r, [&](int64_t k, bool hi, int32_t, int32_t ns) {
+            sizer.count(ns, hi, P.len(ids[r.a_begin + k]), P.len(ids[r.a_begin + (hi ? k + 1 : k)]),
+                        pre[ns]);
+        });
+    }
     for (size_t bi = 0; bi < req.size(); ++bi) {
         const BlockReq& r = req[bi];
         base[bi] = slots;
@@ -362,17 +504,15 @@ int64_t plan_blocks(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& id
         const int32_t bidx = (int32_t)plan.blocks.size() - 1;
         const int64_t* srow = plan.srow.data() + B.srow;
         // residues of the subjects before s, so a query's cells are one product
-        std::vector<int64_t> pre((size_t)r.b_count + 1, 0);
-        for (int64_t s = 0; s < r.b_count; ++s) pre[s + 1] = pre[s] + P.len(ids[r.b_begin + s]);
-        for (int64_t k = 0; k < r.a_count; k += 2) {
-            const bool hi = k + 1 < r.a_count;
-            const int32_t qhi = ids[r.a_begin + (hi ? k + 1 : k)];
-            int32_t ns = (int32_t)r.b_count;
-            if (r.kind == kTri) ns = (int32_t)(hi ? k + 1 : k);
-            for (int64_t q = k; q < k + (hi ? 2 : 1); ++q)
-                plan.cells += P.len(ids[r.a_begin + q]) * pre[(r.kind == kTri) ? q : r.b_count];
-            if (ns > 0) add_tasks(plan, bidx, (int32_t)k, ns, hi, P.len(qhi), srow, target);
-        }
+        pre.assign(1, 0);
+        for (int64_t s = 0; s < r.b_count; ++s)
+            pre.push_back(pre.back() + P.len(ids[r.b_begin + s]));
+        each_query(r, [&](int64_t k, bool hi, int32_t ns_lo, int32_t ns) {
+            const int64_t m_lo = P.len(ids[r.a_begin + k]);
+            const int64_t m_hi = P.len(ids[r.a_begin + (hi ? k + 1 : k)]);
+            plan.cells += m_lo * pre[ns_lo] + (hi ? m_hi * pre[ns] : 0);
+            sizer.add(plan, bidx, (int32_t)k, ns_lo, ns, hi, m_lo, m_hi, srow);
+        });
         if (nslots == 0) {   // keep first_slot strictly usable by the saturated-pair scan
             plan.first_slot.pop_back();
             plan.blocks.pop_back();
@@ -396,7 +536,7 @@ int64_t plan_blocks(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& id
     int64_t maxlen_rows = 1;
     for (size_t s = 0; s + 1 < plan.srow.size(); ++s)
         maxlen_rows = std::max(maxlen_rows, plan.srow[s + 1] - plan.srow[s]);
-    plan.max_warp_rows = 2 * c->rows_per_warp + 2 * maxlen_rows + 2 * target / c->W;
+    plan.max_warp_rows = 4 * (int64_t)c->rows_per_warp + 2 * maxlen_rows;
     return slots;
 }
 
@@ -534,9 +674,10 @@ int score_pairs_int32(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& 
     ENSURE(B_OUT, n, d_out);
     ENSURE(B_FLAGS, kFlagWords, d_flags);
     const int64_t stride = (P.maxlen + 64 + 1) & ~(int64_t)1;
-    const int64_t nslot = std::max<int64_t>((int64_t)c->num_sms * kLongSlots,
-                                            (int64_t)c->num_sms * std::max(1, sw32_ctas_per_sm()));
-    ENSURE(B_BND, nslot * stride, d_bnd);
+    if (c->sw32_occ == 0) c->sw32_occ = std::max(1, sw32_ctas_per_sm());
+    const int64_t grid32 = std::min<int64_t>(n - nlong, (int64_t)c->num_sms * c->sw32_occ);
+    const int64_t grid_long = std::min<int64_t>(nlong, c->num_sms);
+    ENSURE(B_BND, std::max(grid32, grid_long * kLongSlots) * stride, d_bnd);
     int r = copy_in(c, d_pref, lst.data(), lst.size() * sizeof(PairRef), false);
     if (r) return r;
     CUDA_TRY(cudaMemsetAsync(d_flags, 0, kFlagWords * sizeof(int32_t), st));
@@ -554,13 +695,11 @@ int score_pairs_int32(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& 
     a.bnd = d_bnd;
     a.bnd_stride = stride;
     if (nlong > 0) {
-        CUDA_TRY(launch_long_sw32((int)std::min<int64_t>(nlong, c->num_sms), a, d_pref, nlong,
-                                  d_flags + 5, st));
+        CUDA_TRY(launch_long_sw32((int)grid_long, a, d_pref, nlong, d_flags + 5, st));
         c->stats.launches += 1;
     }
     if (n > nlong) {
-        const int grid = (int)std::min<int64_t>(n - nlong, (int64_t)c->num_sms * std::max(1, sw32_ctas_per_sm()));
-        CUDA_TRY(launch_sw32(16, grid, a, d_pref + nlong, (int32_t)(n - nlong), d_flags + 3, st));
+        CUDA_TRY(launch_sw32(16, (int)grid32, a, d_pref + nlong, (int32_t)(n - nlong), d_flags + 3, st));
         c->stats.launches += 1;
     }
     int32_t kerr = 0;
@@ -600,8 +739,8 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
     ENSURE(B_JOBS, n_pairs, d_jobs);
     ENSURE(B_RES, 3 * n_pairs, d_res);
     ENSURE(B_FLAGS, kFlagWords, d_flags);
-    const int occ = std::max(1, cells_wf_ctas_per_sm());
-    const int grid = (int)std::min<int64_t>(n_pairs, (int64_t)c->num_sms * occ);
+    if (c->cells_occ == 0) c->cells_occ = std::max(1, cells_wf_ctas_per_sm());
+    const int grid = (int)std::min<int64_t>(n_pairs, (int64_t)c->num_sms * c->cells_occ);
     const int64_t stride = P.maxlen + 64;
     ENSURE(B_BND, std::max<int64_t>(grid, (int64_t)c->num_sms * kLongSlots) * stride, d_bnd);
     SwArgs a{};
@@ -720,13 +859,15 @@ void allpairs_plan(cm_ctx* c, const Prepared& P, int32_t n_seqs, int64_t part, i
     auto tri = [](int64_t k) { return k * (k - 1) / 2; };
     plan.nslots = tri(k1) - tri(k0);
     plan.pairs = plan.nslots;
-    const int64_t target = (int64_t)c->W * c->rows_per_warp;
-    for (int32_t k = k0; k < k1; k += 2) {
-        const bool hi = (k + 1 < k1);
-        const int32_t ns = hi ? k + 1 : k;
-        const int64_t m_hi = P.hoff[L[hi ? k + 1 : k] + 1] - P.hoff[L[hi ? k + 1 : k]];
-        if (ns > 0) add_tasks(plan, 0, k, ns, hi, m_hi, plan.srow.data(), target);
-    }
+    TaskSizer sizer(c->W, c->num_sms, c->rows_per_warp);
+    for (int step = 0; step < 2; ++step)
+        for (int32_t k = k0; k < k1; k += 2) {
+            const bool hi = (k + 1 < k1);
+            const int32_t ns = hi ? k + 1 : k;
+            const int64_t m_lo = P.len(L[k]), m_hi = P.len(L[hi ? k + 1 : k]);
+            if (step == 0) sizer.count(ns, hi, m_lo, m_hi, plan.srow[ns]);
+            else sizer.add(plan, 0, k, k, ns, hi, m_lo, m_hi, plan.srow.data());
+        }
     {   // cells = sum over pairs of len(a) * len(b)
         int64_t acc = 0, pre = 0;
         for (int32_t k = 0; k < k1; ++k) {
@@ -740,7 +881,7 @@ void allpairs_plan(cm_ctx* c, const Prepared& P, int32_t n_seqs, int64_t part, i
     int64_t maxlen_rows = 1;
     for (int32_t s = 0; s < n_seqs; ++s)
         maxlen_rows = std::max(maxlen_rows, plan.srow[s + 1] - plan.srow[s]);
-    plan.max_warp_rows = 2 * c->rows_per_warp + 2 * maxlen_rows + 2 * target / c->W;
+    plan.max_warp_rows = 4 * (int64_t)c->rows_per_warp + 2 * maxlen_rows;
 
     k0_out = k0;
 }
@@ -876,7 +1017,7 @@ int sw_score_batch(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int32
     std::vector<int32_t> a_ids, b_ids;
     std::vector<int64_t> omap((size_t)n_pairs);
     plan.srow.push_back(0);
-    const int64_t target = (int64_t)c->W * c->rows_per_warp;
+    TaskSizer sizer(c->W, c->num_sms, c->rows_per_warp);
     int64_t slot = 0;
     for (size_t g0 = 0; g0 < ord.size();) {
         size_t g1 = g0;
@@ -906,9 +1047,13 @@ int sw_score_batch(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int32
         }
         plan.first_slot.push_back(B.out_base);
         plan.blocks.push_back(B);
-        add_tasks(plan, (int32_t)plan.blocks.size() - 1, 0, B.nb, false, ma,
-                  plan.srow.data() + B.srow, target);
+        sizer.count(B.nb, false, ma, ma, plan.srow.back() - plan.srow[B.srow]);
         g0 = g1;
+    }
+    for (size_t b = 0; b < plan.blocks.size(); ++b) {
+        const SwBlock& B = plan.blocks[b];
+        const int64_t ma = P.len(a_ids[B.a_ids]);
+        sizer.add(plan, (int32_t)b, 0, B.nb, B.nb, false, ma, ma, plan.srow.data() + B.srow);
     }
     for (auto& B : plan.blocks) B.b_ids += (int64_t)a_ids.size();
     plan.ids = a_ids;
@@ -919,7 +1064,7 @@ int sw_score_batch(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int32
     int64_t maxlen_rows = 0;
     for (size_t s = 0; s + 1 < plan.srow.size(); ++s)
         maxlen_rows = std::max(maxlen_rows, plan.srow[s + 1] - plan.srow[s]);
-    plan.max_warp_rows = 2 * c->rows_per_warp + 2 * maxlen_rows + 2 * target / c->W;
+    plan.max_warp_rows = 4 * (int64_t)c->rows_per_warp + 2 * maxlen_rows;
 
     int64_t* d_omap;
     ENSURE(B_OMAP, n_pairs, d_omap);

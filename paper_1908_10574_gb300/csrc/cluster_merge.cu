@@ -704,7 +704,6 @@ int Driver::score_ranked(const std::vector<Merge>& ms, const std::vector<char>& 
     CUDA_TRY(cudaMemcpyAsync(tot.data(), d_tot, tot.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     c->stats.launches += 1;
-    const int64_t target = (int64_t)c->W * c->rows_per_warp;
     for (int32_t l0 = 0; l0 < nl;) {
         int32_t l1 = l0;
         int64_t rows = 0;
@@ -714,6 +713,16 @@ int Driver::score_ranked(const std::vector<Merge>& ms, const std::vector<char>& 
         plan.total_rows = rows;
         std::vector<int64_t> first;
         int64_t g = 0, rowbase = 0, slots = 0;
+        TaskSizer sizer(c->W, c->num_sms, c->rows_per_warp);
+        auto query_lens = [&](const LMeta& L) {
+            const auto& cs1 = sets[ms[L.m].left];
+            const int64_t a = P.len(arena[cs1[L.op == kKeepBOnly ? L.b : L.a]].rep);
+            return std::make_pair(a, L.op == kKeepAnd ? P.len(arena[cs1[L.b]].rep) : a);
+        };
+        for (int32_t l = l0; l < l1; ++l) {
+            const std::pair<int64_t, int64_t> m = query_lens(meta[l]);
+            sizer.count((int32_t)meta[l].count, meta[l].op == kKeepAnd, m.first, m.second, tot[2 * l]);
+        }
         for (int32_t l = l0; l < l1; ++l) {
             const LMeta& L = meta[l];
             const auto& cs1 = sets[ms[L.m].left];
@@ -740,8 +749,8 @@ int Driver::score_ranked(const std::vector<Merge>& ms, const std::vector<char>& 
             plan.blocks.push_back(B);
             plan.first_slot.push_back(slots);
             first.push_back(slots);
-            add_tasks(plan, (int32_t)plan.blocks.size() - 1, 0, (int32_t)L.count, pair, P.len(qb),
-                      nullptr, target, tot[2 * l]);
+            sizer.add(plan, (int32_t)plan.blocks.size() - 1, 0, (int32_t)L.count, (int32_t)L.count,
+                      pair, P.len(qa), P.len(qb), nullptr, tot[2 * l]);
             plan.cells += (P.len(qa) + (pair ? P.len(qb) : 0)) * tot[2 * l + 1];
             slots += (int64_t)B.na * L.count;
             g += L.count;
@@ -752,7 +761,7 @@ int Driver::score_ranked(const std::vector<Merge>& ms, const std::vector<char>& 
         plan.n_sub = g;
         plan.nslots = plan.pairs = slots;
         order_tasks(plan);
-        plan.max_warp_rows = 2 * c->rows_per_warp + 2 * stream_rows(P.maxlen) + 2 * target / c->W;
+        plan.max_warp_rows = 4 * (int64_t)c->rows_per_warp + 2 * stream_rows(P.maxlen);
         int32_t* d_ids;
         int64_t* d_srow;
         ENSURE(B_IDS, nA + g, d_ids);

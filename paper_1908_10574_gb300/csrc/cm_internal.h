@@ -76,7 +76,19 @@ struct SwTask {
     int32_t npass;      // column passes of SEG*R columns
     int32_t hi_valid;   // 0 when the lo query has no partner
     int32_t mode;
-    int32_t pad;
+    int32_t R;          // columns per lane
+};
+
+// One work unit of the single-query launch: a task's passes [pass, pass_end).  A unit with all
+// passes runs them one after another over its warp's boundary slot.  A unit of one pass of
+// several (a pipelined task: its passes are consecutive units) reads and then overwrites, row
+// by row, the boundary column that the unit before it writes at piped + bnd_row.
+struct SwUnit {
+    int32_t block, k, s0, s1;
+    int32_t npass, pass, pass_end;
+    int32_t mode, R;
+    int32_t rows;       // pipelined: rows of the boundary column
+    int64_t bnd_row;    // pipelined: its first row in SwArgs::piped, else -1
 };
 
 struct SwArgs {
@@ -86,6 +98,10 @@ struct SwArgs {
     const SwTask* tasks;
     int32_t ntasks;
     int32_t* task_counter;      // zeroed before launch
+    const struct SwUnit* units; // single-query launch: its work units (instead of tasks)
+    const int32_t* ranges;      // ... first unit of each CTA (grid + 1)
+    int32_t* progress;          // ... boundary row groups written by each unit (zeroed)
+    uint2* piped;               // ... boundary columns of the pipelined units
     const int32_t* ids;         // id pool
     const uint8_t* streams;     // stream pool
     const int64_t* srows;       // row pool
@@ -138,6 +154,14 @@ struct KeptList {
 // ---- launchers (sw16.cu) ---------------------------------------------------------------
 int sw16_ctas_per_sm(int R, int W, int mode);
 cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st);
+// Every single-query task (kModeTwo, kModeTwo16; any tile width) in one launch of `grid` CTAs of
+// `warps` warps, a unit per warp at a time; CTA b owns the units [ranges[b], ranges[b + 1]),
+// task_counter[b] is its ticket.  Slots of bnd_stride rows for the units of all passes are
+// at bnd, one per warp.  Weak: a build with its own launch_sw16 and without this gets a launch
+// per bin.
+constexpr int kSingleWarps = 12;       // one CTA per SM: shared memory of the profiles
+cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_t st)
+    __attribute__((weak));
 cudaError_t launch_sw32(int R, int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
                         int32_t* counter, cudaStream_t st);
 int sw32_smem_bytes(int R);

@@ -21,7 +21,7 @@ struct Plan {
     std::vector<int64_t> srow;           // global row table over all B subjects (+1)
     std::vector<SwTask> tasks;           // grouped by R, cost descending inside a group
     std::vector<int> task_R;             // launch bin R * 4 + mode per task (parallel to tasks)
-    std::vector<std::pair<int64_t, int>> keys;   // (cost, bin) per task, for ordering
+    std::vector<std::pair<int64_t, int>> keys;   // (cost, bin) per task (parallel to tasks)
     int64_t nslots = 0;
     int64_t cells = 0, cells_padded = 0, pairs = 0;
     int64_t max_warp_rows = 0;
@@ -105,6 +105,7 @@ inline void add_tasks(Plan& P, int32_t block, int32_t k, int32_t ns, bool hi_val
         t.npass = np;
         t.hi_valid = hi_valid ? 1 : 0;
         t.mode = mode;
+        t.R = R;
         const int64_t rows = srow ? srow[e] - srow[s] : rows_total * (e - s) / std::max(ns, 1);
         P.cells_padded += rows * seg * R * np * (single ? 1 : 2);
         P.tasks.push_back(t);
@@ -133,9 +134,77 @@ inline void order_tasks(Plan& P)
     });
     std::vector<SwTask> t2(k.size());
     std::vector<int> r2(k.size());
-    for (size_t i = 0; i < k.size(); ++i) { t2[i] = P.tasks[k[i].i]; r2[i] = P.task_R[k[i].i]; }
+    for (size_t i = 0; i < k.size(); ++i) {
+        t2[i] = P.tasks[k[i].i];
+        r2[i] = P.task_R[k[i].i];
+        P.keys[i] = {k[i].cost, k[i].bin};
+    }
     P.tasks.swap(t2);
     P.task_R.swap(r2);
 }
+
+// Sizes the tasks of a plan.  First pass: count() every query pair (or lone query) with its
+// subjects; second pass, after all are counted: add() makes their tasks.
+//   * A pair of queries shares a CTA of W warps only if it has two subjects for each of the
+//     CTA's streams (W, or 2 W over 16-lane segments); below that the streams, cut at subject
+//     boundaries, are uneven or empty and the CTA waits for its longest one, so the two
+//     queries run as lone queries, one warp each.
+//   * Streams hold rows_per_warp rows in a large plan; in a small one as many as leave two
+//     tasks for every CTA slot of the chip, but no fewer than kMinRows, since a stream also
+//     pays for filling the wavefront (16 or 32 steps of four rows).
+struct TaskSizer {
+    static constexpr int64_t kMinRows = 512;
+    int W;
+    int64_t sms, rows_per_warp;
+    double pair_cost = 0, single_cost = 0;           // rows x columns per lane x passes per stream
+
+    TaskSizer(int W_, int64_t sms_, int64_t rows) : W(W_), sms(sms_), rows_per_warp(rows) {}
+
+    bool paired(int32_t ns, bool hi_valid, int64_t m_hi) const
+    {
+        return hi_valid && ns >= 2 * W * (m_hi <= kSeg16MaxCols ? 2 : 1);
+    }
+    void count(int32_t ns, bool hi_valid, int64_t m_lo, int64_t m_hi, int64_t rows)
+    {
+        if (paired(ns, hi_valid, m_hi)) {
+            pair_cost += cost(choose_tile(m_hi, true), rows);
+        } else {
+            if (hi_valid) single_cost += cost(choose_tile(m_lo, false), rows);
+            single_cost += cost(choose_tile(m_hi, false), rows);
+        }
+    }
+    // queries k and (hi_valid) k + 1 of m_lo and m_hi residues against subjects [0, ns_lo) and
+    // [0, ns); srow / rows as add_tasks
+    void add(Plan& P, int32_t block, int32_t k, int32_t ns_lo, int32_t ns, bool hi_valid,
+             int64_t m_lo, int64_t m_hi, const int64_t* srow, int64_t rows = 0) const
+    {
+        if (paired(ns, hi_valid, m_hi)) {
+            add_tasks(P, block, k, ns, true, m_hi, srow,
+                      W * stream_target(pair_cost / (2.0 * sms * W), choose_tile(m_hi, true)), rows);
+            return;
+        }
+        const double share = single_cost / (2.0 * sms * kSingleWarps);
+        if (hi_valid && ns_lo > 0)
+            add_tasks(P, block, k, ns_lo, false, m_lo, srow,
+                      stream_target(share, choose_tile(m_lo, false)), rows);
+        if (ns > 0)
+            add_tasks(P, block, hi_valid ? k + 1 : k, ns, false, m_hi, srow,
+                      stream_target(share, choose_tile(m_hi, false)), rows);
+    }
+
+private:
+    static double cost(const TileChoice& t, int64_t rows)
+    {
+        return (double)rows * t.R * t.npass / t.spw;
+    }
+    // rows of a stream whose warp then has about `share` of cost (add_tasks multiplies by the
+    // streams per warp and divides by the passes)
+    int64_t stream_target(double share, const TileChoice& t) const
+    {
+        const double rows = share / t.R;
+        return rows >= (double)rows_per_warp ? rows_per_warp
+                                             : std::max(std::min(kMinRows, rows_per_warp), (int64_t)rows);
+    }
+};
 
 }  // namespace cm

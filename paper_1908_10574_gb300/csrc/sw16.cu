@@ -1,5 +1,5 @@
-// Launchers of the Smith-Waterman kernels (templates in sw16_kernel.cuh): the int16x2 kernel
-// dispatch by CTA width, the int32 rescoring kernel and the alignment-cells kernel.
+// Launchers of the Smith-Waterman kernels (templates in sw16_kernel.cuh): the int16x2
+// query-pair kernel by CTA width, the int32 rescoring kernel and the alignment-cells kernel.
 #include "sw16_kernel.cuh"
 
 namespace cm {
@@ -7,18 +7,16 @@ namespace cm {
 #define CM_DECL(w, m)                                                                     \
     cudaError_t launch_sw16_w##w##_m##m(int R, int grid, const SwArgs& a, cudaStream_t st); \
     int sw16_occ_w##w##_m##m(int R);
-CM_DECL(4, 0) CM_DECL(4, 1) CM_DECL(4, 2) CM_DECL(4, 3)
-CM_DECL(8, 0) CM_DECL(8, 1) CM_DECL(8, 2) CM_DECL(8, 3)
-CM_DECL(16, 0) CM_DECL(16, 1) CM_DECL(16, 2) CM_DECL(16, 3)
+CM_DECL(4, 0) CM_DECL(4, 2)
+CM_DECL(8, 0) CM_DECL(8, 2)
+CM_DECL(16, 0) CM_DECL(16, 2)
 #undef CM_DECL
 
 int sw16_ctas_per_sm(int R, int W, int mode)
 {
 #define CM_OCC_CASE(w)                                                                   \
     case w:                                                                              \
-        return mode == kModePair ? sw16_occ_w##w##_m0(R)                                 \
-               : mode == kModeTwo ? sw16_occ_w##w##_m1(R)                                \
-               : mode == kModeSeg16 ? sw16_occ_w##w##_m2(R) : sw16_occ_w##w##_m3(R);
+        return mode == kModePair ? sw16_occ_w##w##_m0(R) : sw16_occ_w##w##_m2(R);
     switch (W) {
     CM_OCC_CASE(4)
     CM_OCC_CASE(8)
@@ -43,12 +41,11 @@ int sw32_ctas_per_sm()
 
 cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st)
 {
+    if (mode != kModePair && mode != kModeSeg16) return cudaErrorInvalidValue;
 #define CM_LAUNCH_CASE(w)                                                                \
     case w:                                                                              \
         return mode == kModePair ? launch_sw16_w##w##_m0(R, grid, a, st)                 \
-               : mode == kModeTwo ? launch_sw16_w##w##_m1(R, grid, a, st)                \
-               : mode == kModeSeg16 ? launch_sw16_w##w##_m2(R, grid, a, st)              \
-                                    : launch_sw16_w##w##_m3(R, grid, a, st);
+                                 : launch_sw16_w##w##_m2(R, grid, a, st);
     switch (W) {
     CM_LAUNCH_CASE(4)
     CM_LAUNCH_CASE(8)

@@ -94,38 +94,10 @@ __device__ __forceinline__ void store_score(const SwArgs& a, const SwBlock& B, i
     if (pass == 0) {
         a.out[slot] = val;
     } else {
-        const int32_t old = a.out[slot];
+        const int32_t old = __ldcg(a.out + slot);    // maybe written by another SM's pass
         if (old != kSat) a.out[slot] = (val == kSat) ? kSat : max(old, val);
     }
 }
-
-// One wavefront segment of SEG lanes (a whole warp, or a half-warp when SEG = 16) against the
-// profile tile of this pass.  Every subject starts on a row that is a multiple of kRowGroup.
-//   pair (TWO = false): the two 16-bit halves are two queries; one subject stream `lo` of
-//     n_lo rows feeds both.
-//   single query (TWO = true): both halves hold the same query; the lo half runs stream `lo`
-//     (n_lo rows), the hi half stream `hi` (n_hi rows).  The profile then carries the score in
-//     its low half only, and the packed score word of a column is hi_row * 2^16 + lo_row (one
-//     multiply-add on the FMA pipe).
-// A step covers NR consecutive rows of each stream; row q of the step trails row q-1 by one
-// column inside the lane, so the NR rows form independent dependency chains and the step's
-// fixed costs (shuffles, residue and flag handling) are shared by NR rows.  The segment's
-// last lane writes one score per finished subject per half.  All lanes of the warp run
-// `nrows_max` rows (the warp's longest stream); shorter streams step through pad rows
-// meanwhile.  Multi-pass tiles (boundary columns in `bnd`) use SEG = 32 only.
-// Rows per step: four (a row group) in the pair modes.  The single-query modes carry a second
-// subject stream (a second residue-row lookup per row) and fit four rows into the register
-// budget only for narrow tiles: four up to 7 columns per lane in 16-lane segments, two up
-// to 16 columns, one above (the host keeps single-query tiles at <= 16 columns per lane).
-template <int R, int SEG, bool TWO>
-struct RowsPerStep {
-    static constexpr int value = !TWO ? 4 : (SEG == 16 && R <= 7) ? 4 : (R <= 16 ? 2 : 1);
-};
-
-template <int NR> struct RowWord;
-template <> struct RowWord<1> { typedef uint8_t type; };
-template <> struct RowWord<2> { typedef uint16_t type; };
-template <> struct RowWord<4> { typedef uint32_t type; };
 
 // load the profile words of columns [c, c + 4) of one row (fewer at the tile's right edge;
 // the lane's row segment always holds whole 16-byte units)
@@ -143,34 +115,38 @@ __device__ __forceinline__ void load_cols(const uint32_t* p, int c, uint32_t (&v
     }
 }
 
-template <int R, int SEG, bool TWO>
+// One wavefront segment of SEG lanes (a whole warp, or a half-warp when SEG = 16) against the
+// profile tile of this pass: the two 16-bit halves are two queries, and the subject stream of
+// n_rows rows (every subject starts on a multiple of kRowGroup) feeds both.  A step covers a
+// row group; row q of the step trails row q-1 by one column inside the lane, so the rows form
+// independent dependency chains and the step's fixed costs (shuffles, residue and flag
+// handling) are shared by them.  The segment's last lane writes one score per finished subject
+// per half.  All lanes of the warp run `nrows_max` rows (the warp's longest stream); shorter
+// streams step through pad rows meanwhile.  Multi-pass tiles (boundary columns in `bnd`) use
+// SEG = 32 only.
+template <int R, int SEG>
 __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
                                           const uint32_t* __restrict__ prof,
-                                          const uint8_t* __restrict__ st_lo, int64_t n_lo,
-                                          const uint8_t* __restrict__ st_hi, int64_t n_hi,
+                                          const uint8_t* __restrict__ stream, int64_t n_rows,
                                           int64_t nrows_max, int pass, int npass,
-                                          uint2* __restrict__ bnd, int32_t s_lo0, int32_t s_hi0,
-                                          int32_t k_lo, int32_t ns_lo, int32_t ns_hi,
-                                          bool hi_valid)
+                                          uint2* __restrict__ bnd, int32_t s0, int32_t k_lo,
+                                          int32_t ns_lo, int32_t ns_hi, bool hi_valid)
 {
     using G = Geo<R, SEG>;
-    constexpr int NR = RowsPerStep<R, SEG, TWO>::value;
-    typedef typename RowWord<NR>::type word_t;
+    constexpr int NR = kRowGroup;
     const int lane = threadIdx.x & (SEG - 1);    // lane within the segment
     const int o = a.gap_open, ge = a.gap_extend, beta = a.beta;
     const uint32_t BETA2 = (uint32_t)beta * 0x10001u;
     const uint32_t BMO2 = (uint32_t)(beta - o) * 0x10001u;   // H - o of an empty prefix; E, F floor
     const uint32_t O2 = (uint32_t)o * 0x10001u;
     const uint32_t NEGE = pack2(-ge, -ge);
-    const uint32_t PADW = (kPadCode * 0x01010101u) >> (32 - 8 * NR);   // kPadCode in every byte
+    constexpr uint32_t PADW = kPadCode * 0x01010101u;
     // boundary records of one step: (H - o, E) of the last column of each of its rows, as
-    // uint4 pairs of rows (one uint2 when a step has one row)
-    constexpr int NB = (NR >= 2) ? NR / 2 : 1;
+    // uint4 pairs of rows
+    constexpr int NB = NR / 2;
     uint4* bnd4 = reinterpret_cast<uint4*>(bnd);
-    const uint32_t CODEMASK = 0x1f1f1f1fu >> (32 - 8 * NR);           // residue code bits
-    uint32_t LASTBITS = 0;
-#pragma unroll
-    for (int q = 0; q < NR; ++q) LASTBITS |= (uint32_t)kLast << (8 * q);
+    constexpr uint32_t CODEMASK = 0x1f1f1f1fu;                        // residue code bits
+    constexpr uint32_t LASTBITS = kLast * 0x01010101u;
 
     // hp[c] holds H - o of the row above (the value both E and F start a gap from, and the
     // diagonal of column c+1 against a profile that carries +o); fp[c] holds F.
@@ -182,43 +158,31 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
 #pragma unroll
     for (int q = 0; q < NR; ++q) { oh[q] = BMO2; oe[q] = BMO2; }
     uint32_t diag0 = BMO2;                        // left H - o of the previous step's last row
-    uint32_t cur = PADW, prev = PADW, cur2 = PADW, prev2 = PADW;
+    uint32_t cur = PADW, prev = PADW;
     uint4 bv[NB];
 #pragma unroll
     for (int q = 0; q < NB; ++q) bv[q] = make_uint4(BMO2, BMO2, BMO2, BMO2);
-    int32_t s_lo = s_lo0, s_hi = s_hi0;
+    int32_t s_next = s0;
     const uint32_t* plane = prof + lane * G::LS;
-    const int nsup = (int)(n_lo / NR);            // a warp stream holds < 2^31 rows
-    const int nsup2 = TWO ? (int)(n_hi / NR) : 0;
+    const int nsup = (int)(n_rows / NR);          // a warp stream holds < 2^31 rows
     const int nsup_max = (int)(nrows_max / NR);
     const int nsteps = nsup_max + SEG - 1;
-    const word_t* stw = reinterpret_cast<const word_t*>(st_lo);
-    const word_t* stw2 = reinterpret_cast<const word_t*>(st_hi);
+    const uint32_t* stw = reinterpret_cast<const uint32_t*>(stream);
 
     for (int t = 0; t < nsteps; ++t) {
         const int j = t & (SEG - 1);
         if (j == 0) {
             const int u = t + lane;
             prev = cur;
-            cur = (u < nsup) ? (uint32_t)stw[u] : PADW;
-            if (TWO) {
-                prev2 = cur2;
-                cur2 = (u < nsup2) ? (uint32_t)stw2[u] : PADW;
-            }
+            cur = (u < nsup) ? stw[u] : PADW;
             if (SEG == 32 && pass > 0) {
-                if constexpr (NR >= 2) {
 #pragma unroll
-                    for (int q = 0; q < NB; ++q)
-                        bv[q] = (u < nsup_max) ? bnd4[u * NB + q] : make_uint4(BMO2, BMO2, BMO2, BMO2);
-                } else {
-                    const uint2 v = (u < nsup_max) ? bnd[u] : make_uint2(BMO2, BMO2);
-                    bv[0] = make_uint4(v.x, v.y, BMO2, BMO2);
-                }
+                for (int q = 0; q < NB; ++q)
+                    bv[q] = (u < nsup_max) ? bnd4[u * NB + q] : make_uint4(BMO2, BMO2, BMO2, BMO2);
             }
         }
         const int src = (j - lane) & (SEG - 1);
         const uint32_t rv = __shfl_sync(kFull, (lane <= j) ? cur : prev, src, SEG);
-        const uint32_t rw = TWO ? __shfl_sync(kFull, (lane <= j) ? cur2 : prev2, src, SEG) : 0u;
         uint32_t hL[NR], eL[NR];
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
@@ -231,10 +195,8 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
             for (int q = 0; q < NB; ++q) {
                 const uint32_t x0 = __shfl_sync(kFull, bv[q].x, j), x1 = __shfl_sync(kFull, bv[q].y, j);
                 if (lane == 0) { hL[2 * q] = x0; eL[2 * q] = x1; }
-                if constexpr (NR >= 2) {
-                    const uint32_t x2 = __shfl_sync(kFull, bv[q].z, j), x3 = __shfl_sync(kFull, bv[q].w, j);
-                    if (lane == 0) { hL[2 * q + 1] = x2; eL[2 * q + 1] = x3; }
-                }
+                const uint32_t x2 = __shfl_sync(kFull, bv[q].z, j), x3 = __shfl_sync(kFull, bv[q].w, j);
+                if (lane == 0) { hL[2 * q + 1] = x2; eL[2 * q + 1] = x3; }
             }
         } else if (lane == 0) {
 #pragma unroll
@@ -246,32 +208,19 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
 #pragma unroll
         for (int q = 1; q < NR; ++q) dg[q] = hL[q - 1];
         diag0 = hL[NR - 1];
-        if (!TWO) {
-            if (rv & kFirst) {                    // a subject starts at the step's first row
+        if (rv & kFirst) {                        // a subject starts at the step's first row
 #pragma unroll
-                for (int k = 0; k < R; ++k) { hp[k] = BMO2; fp[k] = BMO2; }
-                best = BETA2;
-                dg[0] = BMO2;
-            }
-        } else if ((rv | rw) & kFirst) {          // per half: whose stream starts a subject
-            const uint32_t keep = ((rv & kFirst) ? 0u : 0x0000ffffu) | ((rw & kFirst) ? 0u : 0xffff0000u);
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                hp[k] = (hp[k] & keep) | (BMO2 & ~keep);
-                fp[k] = (fp[k] & keep) | (BMO2 & ~keep);
-            }
-            best = (best & keep) | (BETA2 & ~keep);
-            dg[0] = (dg[0] & keep) | (BMO2 & ~keep);
+            for (int k = 0; k < R; ++k) { hp[k] = BMO2; fp[k] = BMO2; }
+            best = BETA2;
+            dg[0] = BMO2;
         }
         // profile row of each residue: one mask takes the flags off all NR bytes, one byte
         // permute moves a code to the low byte (the stream writer keeps codes <= kPadCode)
-        const uint32_t rc = rv & CODEMASK, rc2 = TWO ? (rw & CODEMASK) : 0u;
+        const uint32_t rc = rv & CODEMASK;
         const uint32_t* prow[NR];
-        const uint32_t* prow2[NR];
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
             prow[q] = plane + __byte_perm(rc, 0u, 0x4440u | q) * G::ROWW;
-            if (TWO) prow2[q] = plane + __byte_perm(rc2, 0u, 0x4440u | q) * G::ROWW;
             h[q] = hL[q];
             e[q] = eL[q];
         }
@@ -288,16 +237,7 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
             for (int q = 0; q < NR; ++q) {
                 const int c = k - q;
                 if (c < 0 || c >= R) continue;
-                if ((c & 3) == 0) {               // next (up to) four profile columns of row q
-                    load_cols<R>(prow[q], c, sq[q]);
-                    if (TWO) {
-                        uint32_t v2[4];
-                        load_cols<R>(prow2[q], c, v2);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (c + u < R) sq[q][u] = v2[u] * 0x10000u + sq[q][u];
-                    }
-                }
+                if ((c & 3) == 0) load_cols<R>(prow[q], c, sq[q]);   // next profile columns
                 e[q] = __viaddmax_s16x2(e[q], NEGE, h[q]);
                 const uint32_t f = __viaddmax_s16x2(fp[c], NEGE, hp[c]);
                 const uint32_t d = __viaddmax_s16x2(dg[q], sq[q][c & 3], BETA2);
@@ -317,47 +257,29 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
         if (lane == SEG - 1) {
             const int32_t lo = (int32_t)(int16_t)(out_acc & 0xffffu);
             const int32_t hi = (int32_t)(int16_t)(out_acc >> 16);
-            if (!TWO) {
-                if (rv & LASTBITS) {
-                    const int32_t s = s_lo++;
-                    if (s < ns_lo) store_score(a, B, k_lo, s, lo, pass);
-                    if (hi_valid && s < ns_hi) store_score(a, B, k_lo + 1, s, hi, pass);
-                }
-            } else {
-                if (rv & LASTBITS) {
-                    const int32_t s = s_lo++;
-                    if (s < ns_lo) store_score(a, B, k_lo, s, lo, pass);
-                }
-                if (rw & LASTBITS) {
-                    const int32_t s = s_hi++;
-                    if (s < ns_lo) store_score(a, B, k_lo, s, hi, pass);
-                }
+            if (rv & LASTBITS) {
+                const int32_t s = s_next++;
+                if (s < ns_lo) store_score(a, B, k_lo, s, lo, pass);
+                if (hi_valid && s < ns_hi) store_score(a, B, k_lo + 1, s, hi, pass);
             }
         }
         if (SEG == 32 && lane == 31 && pass + 1 < npass && t >= 31) {
-            if constexpr (NR >= 2) {
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
-                    bnd4[(t - 31) * NB + q] = make_uint4(oh[2 * q], oe[2 * q], oh[2 * q + 1], oe[2 * q + 1]);
-            } else {
-                bnd[t - 31] = make_uint2(oh[0], oe[0]);
-            }
+            for (int q = 0; q < NB; ++q)
+                bnd4[(t - 31) * NB + q] = make_uint4(oh[2 * q], oe[2 * q], oh[2 * q + 1], oe[2 * q + 1]);
         }
     }
 }
 
-// Persistent int16x2 kernel.  MODE kModePair: a query pair (two 16-bit halves) per task, one
-// subject stream per warp over 32 lanes.  kModeTwo: one query, two subject streams in the two
-// halves of each warp.  kModeSeg16: a query pair, two subject streams per warp, one per
-// half-warp segment of 16 lanes.  kModeTwo16: one query, four subject streams per warp (two
-// 16-lane segments x two halves).  The 16-lane modes serve short queries (16 lanes x R).
+// Persistent int16x2 kernel of the query pairs (two 16-bit halves).  MODE kModePair: one
+// subject stream per warp over 32 lanes.  kModeSeg16: two subject streams per warp, one per
+// half-warp segment of 16 lanes, for short queries (16 lanes x R).  Lone queries: sw16_single.cu.
 template <int R, int W, int MODE>
 __global__ void __launch_bounds__(W * 32, 16 / W)
 sw16_kernel(const __grid_constant__ SwArgs a)
 {
-    constexpr bool TWO = (MODE == kModeTwo || MODE == kModeTwo16);
-    constexpr int SEG = (MODE == kModeSeg16 || MODE == kModeTwo16) ? 16 : 32;
-    constexpr int SPW = (MODE == kModePair) ? 1 : (MODE == kModeTwo16) ? 4 : 2;   // streams per warp
+    constexpr int SEG = MODE == kModeSeg16 ? 16 : 32;
+    constexpr int SPW = MODE == kModeSeg16 ? 2 : 1;            // streams per warp
     using G = Geo<R, SEG>;
     extern __shared__ __align__(16) uint8_t smem[];
     uint32_t* prof = reinterpret_cast<uint32_t*>(smem);
@@ -380,10 +302,10 @@ sw16_kernel(const __grid_constant__ SwArgs a)
         const SwBlock B = a.blocks[T.block];
         const int32_t* A_ids = a.ids + B.a_ids;
         const int32_t q_lo = A_ids[T.k];
-        const int32_t q_hi = (!TWO && T.hi_valid) ? A_ids[T.k + 1] : q_lo;
+        const int32_t q_hi = T.hi_valid ? A_ids[T.k + 1] : q_lo;
         const int64_t qoff_lo = a.off[q_lo], m_lo = a.off[q_lo + 1] - qoff_lo;
         const int64_t qoff_hi = a.off[q_hi];
-        const int64_t m_hi = (!TWO && T.hi_valid) ? a.off[q_hi + 1] - qoff_hi : 0;
+        const int64_t m_hi = T.hi_valid ? a.off[q_hi + 1] - qoff_hi : 0;
         const int32_t ns_lo = (B.kind == kTri) ? T.k : B.nb;
         const int32_t ns_hi = (B.kind == kTri) ? T.k + 1 : B.nb;
         const int64_t* srow = a.srows + B.srow;
@@ -398,19 +320,14 @@ sw16_kernel(const __grid_constant__ SwArgs a)
             sb[i] = nearest_boundary(srow, T.s0, T.s1, R0 + (R1 - R0) * (warp * SPW + i) / NS);
             if (i > 0) nmax = max(nmax, srow[sb[i]] - srow[sb[i - 1]]);
         }
-        // this lane's streams: index of the lo stream among the warp's SPW
-        const int seg = (SEG == 16) ? (lane >> 4) : 0;
-        const int i_lo = TWO ? 2 * seg : seg;
-        const int32_t slo0 = sb[i_lo], slo1 = sb[i_lo + 1];
-        const int32_t shi0 = TWO ? sb[i_lo + 1] : slo1, shi1 = TWO ? sb[i_lo + 2] : slo1;
-        int64_t n_lo = srow[slo1] - srow[slo0];
-        int64_t n_hi = srow[shi1] - srow[shi0];
+        const int seg = (SEG == 16) ? (lane >> 4) : 0;          // this lane's stream
+        const int32_t st0 = sb[seg], st1 = sb[seg + 1];
+        int64_t n_rows = srow[st1] - srow[st0];
         if (T.npass > 1 && (SEG == 16 || nmax > a.bnd_stride)) {
             if (lane == 0) atomicExch(a.err, 1);      // boundary buffer too small: refuse
-            n_lo = n_hi = nmax = 0;
+            n_rows = nmax = 0;
         }
-        const uint8_t* st_lo = a.streams + B.stream + srow[slo0];
-        const uint8_t* st_hi = a.streams + B.stream + srow[shi0];
+        const uint8_t* stream = a.streams + B.stream + srow[st0];
 
         for (int pass = 0; pass < T.npass; ++pass) {
             const int64_t c0 = (int64_t)pass * G::COLS;
@@ -423,17 +340,17 @@ sw16_kernel(const __grid_constant__ SwArgs a)
                 const int x = i / G::COLS, c = i - x * G::COLS;
                 const int ln = c / R, k = c - ln * R;
                 const int ql = qres[c], qh = qres[G::COLS + c];
-                int sl = kSpad, sh = TWO ? 0 : kSpad;
+                int sl = kSpad, sh = kSpad;
                 if (x != kPadCode) {          // +o: the DP keeps H - o as its diagonal input
                     if (ql != kPadCode) sl = (B.swap ? s_mat[x * kAlpha + ql] : s_mat[ql * kAlpha + x]) + a.gap_open;
-                    if (!TWO && qh != kPadCode) sh = (B.swap ? s_mat[x * kAlpha + qh] : s_mat[qh * kAlpha + x]) + a.gap_open;
+                    if (qh != kPadCode) sh = (B.swap ? s_mat[x * kAlpha + qh] : s_mat[qh * kAlpha + x]) + a.gap_open;
                 }
                 prof[x * G::ROWW + ln * G::LS + k] = pack2(sl, sh);
             }
             __syncthreads();
             if (nmax > 0)
-                warp_dp16<R, SEG, TWO>(a, B, prof, st_lo, n_lo, st_hi, n_hi, nmax, pass, T.npass,
-                                       bnd, slo0, shi0, T.k, ns_lo, ns_hi, T.hi_valid != 0);
+                warp_dp16<R, SEG>(a, B, prof, stream, n_rows, nmax, pass, T.npass, bnd, st0, T.k,
+                                  ns_lo, ns_hi, T.hi_valid != 0);
             __syncthreads();
         }
     }

@@ -3,4 +3,4 @@
 #define CM_MODE 2
 #define CM_LAUNCH launch_sw16_w16_m2
 #define CM_OCC sw16_occ_w16_m2
-#include "sw16_inst.cuh"
+#include "sw16_pair_inst.cuh"

@@ -3,4 +3,4 @@
 #define CM_MODE 0
 #define CM_LAUNCH launch_sw16_w8_m0
 #define CM_OCC sw16_occ_w8_m0
-#include "sw16_inst.cuh"
+#include "sw16_pair_inst.cuh"
