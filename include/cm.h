@@ -187,9 +187,9 @@ int sw_allpairs(cm_ctx *ctx, const uint8_t *seqs, const int64_t *offsets, int32_
  * that span it is the global affine alignment of the two substrings (same gap costs), which
  * scores the local optimum; among equal-scoring ones the traceback from the end takes an
  * aligned pair first, then I, then D, and a gap's opening before its extension.  If
- * *n_ops > ops_capacity nothing is written and CM_ERR_CAPACITY is returned.  One GPU thread
- * aligns one pair (a p x q byte matrix of choices per pair in device scratch): meant for the
- * similar pairs of a clustering, not for all-against-all. */
+ * *n_ops > ops_capacity nothing is written and CM_ERR_CAPACITY is returned.  One GPU warp
+ * aligns one pair (half a byte of choices per cell of its span in device scratch, 1 GB of it at
+ * a time): meant for the similar pairs of a clustering, not for all-against-all. */
 int sw_align_batch(cm_ctx *ctx, const uint8_t *seqs, const int64_t *offsets, int32_t n_seqs,
                    const int32_t *pairs, int64_t n_pairs, const int8_t *matrix,
                    int32_t gap_open, int32_t gap_extend, int32_t *cells_out,

@@ -210,7 +210,12 @@ class Context:
         cells = np.empty((npairs, 5), dtype=np.int32)
         offs = np.empty(npairs + 1, dtype=np.int64)
         total = ctypes.c_int64(0)
+        # room for a run every four residues; a call that needs more says so and runs again
         cap = 0
+        if n > 0 and npairs > 0:
+            lens = np.clip(np.diff(offsets), 0, 1 << 28)
+            shorter = lens[np.where((pairs >= 0) & (pairs < n), pairs, 0)].min(axis=1)
+            cap = min(npairs + int(shorter.sum()) // 4, 1 << 26)
         for _attempt in range(2):
             runs = np.empty(max(cap, 1), dtype=np.int32)
             code = _L.lib().sw_align_batch(self._h, _ptr(seqs), _ptr(offsets), n, _ptr(pairs),

@@ -29,6 +29,7 @@
 // and a launch per tile: 50,000 pairs of 5,000 proteins (ten subjects per query) 26.6 -> 9.4 ms
 // per call, the kernel 20+ -> 4.9 ms at 59 % ALU; one query against 200 proteins 0.84 -> 0.37 ms;
 // 24 pairs of 8,000-12,000 residues 84.5 -> 13.0 ms (9.8 ms of it the int32 rescoring).
+#include "progress.cuh"
 #include "sw16_kernel.cuh"
 
 namespace cm {
@@ -58,34 +59,6 @@ struct SingleArgs {
     int32_t* done_out;            // ... and by this one (null: nobody waits)
     int32_t* err;
 };
-
-constexpr int kPollLimit = 1 << 24;               // polls of ~100 ns before a wait gives up
-
-// waits (one lane polls) until `need` row groups of the boundary column are written; gives up
-// after kPollLimit polls, or when another wait has
-__device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, const int32_t* err)
-{
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) {
-        for (int polls = 0;; ++polls) {
-            int32_t v;
-            asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
-            if (v >= need) break;
-            if (polls >= kPollLimit ||
-                ((polls & 1023) == 1023 && *reinterpret_cast<const volatile int32_t*>(err) != 0)) {
-                ok = 0;
-                break;
-            }
-            __nanosleep(100);
-        }
-    }
-    return __shfl_sync(kFull, ok, 0) != 0;
-}
-
-__device__ __forceinline__ void publish_groups(int32_t* done, int32_t groups)
-{
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(done), "r"(groups) : "memory");
-}
 
 // packed score of two streams: byte j of each word, sign-extended to 16 bits
 template <int J>
