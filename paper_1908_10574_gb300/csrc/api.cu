@@ -717,68 +717,119 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
     if (n_pairs == 0) return CM_OK;
     if (n_pairs >= ((int64_t)1 << 31)) return fail(c, CM_ERR_ARG, "n_pairs must be < 2^31");
     const cudaStream_t st = c->stream;
-    // jobs longest first (the persistent warps claim them in order), pad = the pair's index
-    // long jobs (many column passes) first, for whole CTAs; the rest longest first
+    // long jobs first (a launch of their own, its waits bounded by cm_set_wait_limit), then the
+    // rest, each longest first; pad = the pair's index
     auto is_long = [](const CellJob& x) { return x.n >= kLongMinCols && x.m >= kLongMinRows; };
-    auto lpt = [&](std::vector<CellJob>& v) {
-        std::stable_sort(v.begin(), v.end(), [&](const CellJob& x, const CellJob& y) {
-            const bool lx = is_long(x), ly = is_long(y);
-            if (lx != ly) return lx;
-            return (int64_t)x.m * x.n > (int64_t)y.m * y.n;
-        });
-    };
     std::vector<CellJob> jobs((size_t)n_pairs);
-    for (int64_t k = 0; k < n_pairs; ++k) {
-        const int32_t x = hp[2 * k], y = hp[2 * k + 1];
-        jobs[k] = CellJob{x, y, (int32_t)P.len(x), (int32_t)P.len(y), 0, (int32_t)k};
+    {
+        std::vector<std::pair<int64_t, int32_t>> key((size_t)n_pairs);
+        for (int64_t k = 0; k < n_pairs; ++k) {
+            const int64_t m = P.len(hp[2 * k]), n = P.len(hp[2 * k + 1]);
+            key[k] = {-m * n, (int32_t)k};
+        }
+        std::sort(key.begin(), key.end());
+        for (int64_t q = 0; q < n_pairs; ++q) {
+            const int32_t k = key[q].second, x = hp[2 * (int64_t)k], y = hp[2 * (int64_t)k + 1];
+            jobs[q] = CellJob{x, y, (int32_t)P.len(x), (int32_t)P.len(y), 0, k};
+        }
+        std::stable_partition(jobs.begin(), jobs.end(), is_long);
     }
-    lpt(jobs);
+    int32_t max_score = 0;
+    for (int i = 0; i < kAlpha * kAlpha; ++i) max_score = std::max<int32_t>(max_score, P.mat[i]);
     CellJob* d_jobs;
     int32_t *d_res, *d_flags;
-    uint2* d_bnd;
     ENSURE(B_JOBS, n_pairs, d_jobs);
     ENSURE(B_RES, 3 * n_pairs, d_res);
-    ENSURE(B_FLAGS, kFlagWords, d_flags);
-    if (c->cells_occ == 0) c->cells_occ = std::max(1, cells_wf_ctas_per_sm());
-    const int grid = (int)std::min<int64_t>(n_pairs, (int64_t)c->num_sms * c->cells_occ);
-    const int64_t stride = P.maxlen + 64;
-    ENSURE(B_BND, std::max<int64_t>(grid, (int64_t)c->num_sms * kLongSlots) * stride, d_bnd);
     SwArgs a{};
     a.db = P.db;
     a.off = P.off;
-    a.bnd = d_bnd;
-    a.bnd_stride = stride;
-    a.err = d_flags + 1;
     a.wait_limit = c->wait_limit;
     std::memcpy(a.mat, P.mat, sizeof(a.mat));
     a.gap_open = P.g1;
     a.gap_extend = P.ge;
+    a.num_sms = c->num_sms;
+    // All jobs (nlong long ones first), in rounds whose boundary columns hold at most kPipedRows
+    // rows; a round's long jobs run on the auxiliary stream beside its other ones, so the few
+    // warps of their pipelines do not have the chip to themselves.
+    auto run_jobs = [&](int32_t nlong) -> int {
+        const int32_t nj = (int32_t)jobs.size();
+        for (int32_t q = 0; q < nj;) {
+            std::vector<CellUnit> units;
+            int64_t rows = 0, ulong_ = 0;
+            bool huge = false;
+            int32_t e = q;
+            for (; e < nj; ++e) {
+                const CellJob& J = jobs[e];
+                const int32_t strips = cell_strips(J.m, J.n), first = e < nlong ? q : std::max(q, nlong);
+                const int64_t more = strips > 1 ? stream_rows(J.m) : 0;   // whole row groups
+                if (e > q && (rows + more > kPipedRows || (int64_t)units.size() + strips > INT32_MAX)) break;
+                huge = huge || std::min<int64_t>(J.m, J.n) * max_score >= kWaveScoreLimit;
+                for (int32_t t = 0; t < strips; ++t)
+                    units.push_back({e - first, t, e < nlong ? c->wait_limit : kPollLimit, 0, rows});
+                rows += more;
+                if (e < nlong) ulong_ = (int64_t)units.size();
+            }
+            int r;
+            const int64_t nu = (int64_t)units.size();
+            CellUnit* d_units;
+            int4* d_best;
+            uint2* d_bnd;
+            ENSURE(B_FLAGS, kFlagWords + nu, d_flags);
+            ENSURE(B_UNITS, nu, d_units);
+            ENSURE(B_BEST, nu, d_best);
+            const int32_t lend = std::min(std::max(q, nlong), e);      // [q, lend) long, [lend, e) not
+            const int huge_grid = (int)std::min<int64_t>(std::max(lend - q, 1), c->num_sms);
+            const int64_t huge_rows = huge ? (int64_t)huge_grid * kLongSlots * (P.maxlen + 64) : 0;
+            ENSURE(B_BND, rows + huge_rows, d_bnd);
+            if ((r = copy_in(c, d_units, units.data(), units.size() * sizeof(CellUnit), false))) return r;
+            CUDA_TRY(cudaMemsetAsync(d_flags, 0, (kFlagWords + nu) * sizeof(int32_t), st));
+            a.err = d_flags + 1;
+            auto part = [&](int32_t j0, int32_t j1, int64_t u0, int64_t u1, bool lng) {
+                const bool hg = lng && huge;
+                a.bnd = d_bnd + (hg ? rows : 0);
+                a.bnd_stride = P.maxlen + 64;
+                a.cell_units = hg ? nullptr : d_units + u0;
+                a.ncells = (int32_t)(u1 - u0);
+                a.progress = d_flags + kFlagWords + u0;
+                a.cell_best = d_best + u0;
+                int32_t* out = d_res + 3 * (int64_t)j0;
+                c->stats.launches += 1;
+                return lng ? launch_long_cells(huge_grid, a, d_jobs + j0, j1 - j0, d_flags + 6, out, c->aux)
+                           : launch_cells_wf((int)std::min<int64_t>(j1 - j0, c->num_sms), a, d_jobs + j0,
+                                             j1 - j0, d_flags + 4, out, st);
+            };
+            cudaError_t le = cudaSuccess;
+            if (lend > q) {
+                CUDA_TRY(cudaEventRecord(c->fork, st));
+                CUDA_TRY(cudaStreamWaitEvent(c->aux, c->fork, 0));
+                le = part(q, lend, 0, ulong_, true);
+            }
+            if (e > lend && le == cudaSuccess) le = part(lend, e, ulong_, nu, false);
+            if (lend > q) {                       // no launch of this call outlives it
+                CUDA_TRY(cudaEventRecord(c->join, c->aux));
+                CUDA_TRY(cudaStreamWaitEvent(st, c->join, 0));
+            }
+            CUDA_TRY(le);
+            int32_t kerr = 0;
+            CUDA_TRY(cudaMemcpyAsync(&kerr, a.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            CUDA_TRY(cudaStreamSynchronize(st));
+            if (kerr == 2) return fail(c, CM_ERR_TIMEOUT, "a long-pair pipeline wait gave up");
+            if (kerr) return fail(c, CM_ERR_INTERNAL, "cells kernel bounds check fired");
+            q = e;
+        }
+        return CM_OK;
+    };
     std::vector<int32_t> fwd((size_t)n_pairs * 3);
     for (int dir = 0; dir < 2; ++dir) {
         int r = copy_in(c, d_jobs, jobs.data(), jobs.size() * sizeof(CellJob), false);
         if (r) return r;
-        CUDA_TRY(cudaMemsetAsync(d_flags, 0, kFlagWords * sizeof(int32_t), st));
         int32_t nlong = 0;
         while (nlong < (int32_t)jobs.size() && is_long(jobs[nlong])) ++nlong;
-        if (nlong > 0) {
-            CUDA_TRY(launch_long_cells((int)std::min<int64_t>(nlong, c->num_sms), a, d_jobs, nlong,
-                                       d_flags + 6, d_res, st));
-            c->stats.launches += 1;
-        }
-        const int32_t nshort = (int32_t)jobs.size() - nlong;
-        if (nshort > 0) {
-            CUDA_TRY(launch_cells_wf((int)std::min<int64_t>(grid, nshort), a, d_jobs + nlong, nshort,
-                                     d_flags + 4, d_res + 3 * (int64_t)nlong, st));
-            c->stats.launches += 1;
-        }
+        if ((r = run_jobs(nlong))) return r;
         std::vector<int32_t> res(jobs.size() * 3);
-        int32_t kerr = 0;
         CUDA_TRY(cudaMemcpyAsync(res.data(), d_res, res.size() * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, st));
-        CUDA_TRY(cudaMemcpyAsync(&kerr, d_flags + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         CUDA_TRY(cudaStreamSynchronize(st));
-        if (kerr == 2) return fail(c, CM_ERR_TIMEOUT, "a long-pair pipeline wait gave up");
-        if (kerr) return fail(c, CM_ERR_INTERNAL, "cells kernel bounds check fired");
         if (dir == 0) {
             fwd = res;
             std::vector<CellJob> rev;
@@ -792,7 +843,7 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
                                           fwd[3 * q + 2] + 1, 1, (int32_t)k});
             }
             if (rev.empty()) break;
-            lpt(rev);
+            std::stable_partition(rev.begin(), rev.end(), is_long);   // about longest first still
             jobs.swap(rev);
         } else {
             for (size_t q = 0; q < jobs.size(); ++q) {

@@ -91,6 +91,8 @@ struct SwUnit {
     int64_t bnd_row;    // pipelined: its first row in SwArgs::piped, else -1
 };
 
+struct CellUnit;
+
 struct SwArgs {
     const uint8_t* db;          // residue codes of all sequences
     const int64_t* off;         // n_seqs+1 offsets
@@ -102,6 +104,10 @@ struct SwArgs {
     const int32_t* ranges;      // ... first unit of each CTA (grid + 1)
     int32_t* progress;          // ... boundary row groups written by each unit (zeroed)
     uint2* piped;               // ... boundary columns of the pipelined units
+    const CellUnit* cell_units; // alignment-cells launch: its units (null: the huge-score kernel)
+    int32_t ncells;
+    int32_t num_sms;
+    int4* cell_best;            // ... best cell up to each unit's strip
     const int32_t* ids;         // id pool
     const uint8_t* streams;     // stream pool
     const int64_t* srows;       // row pool
@@ -137,6 +143,28 @@ struct CellJob {
     int32_t pad;
 };
 
+// Strips of the alignment-cells wavefront (wave32.cuh): at most 32 lanes x kWaveMaxR columns of
+// b, of equal width; a unit of its launch is one strip of one job.
+constexpr int kWaveMaxR = 8;           // columns per lane: two profile words
+constexpr int64_t kWaveScoreLimit = (int64_t)1 << 28;
+constexpr int32_t kPollLimit = 1 << 24;   // polls of ~100 ns before a device wait gives up
+inline __host__ __device__ int32_t wave_strips(int64_t n)
+{
+    return n <= 0 ? 1 : (int32_t)((n + 32 * kWaveMaxR - 1) / (32 * kWaveMaxR));
+}
+inline __host__ __device__ int32_t wave_R(int64_t n)
+{
+    const int64_t per = (n + wave_strips(n) - 1) / wave_strips(n);
+    return per <= 0 ? 1 : (int32_t)((per + 31) / 32);
+}
+inline __host__ __device__ int32_t cell_strips(int64_t m, int64_t n) { return m <= 0 ? 1 : wave_strips(n); }
+struct CellUnit {
+    int32_t job, strip;
+    int32_t limit;                     // polls of its wait for the strip before
+    int32_t pad;
+    int64_t bnd_row;                   // first row of the job's boundary column in SwArgs::bnd
+};
+
 // One subject list of a ranked block, selected by bitmap rows of the ranker's pair selection:
 // op 0 = row a, 1 = row a AND row b, 2 = row a AND NOT row b, 3 = row b AND NOT row a.  Bit i
 // of a row selects subject reps[b0 + i].  The list's subjects become global subjects g0 ..,
@@ -165,13 +193,16 @@ cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_
 cudaError_t launch_sw32(int R, int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
                         int32_t* counter, cudaStream_t st);
 int sw32_smem_bytes(int R);
-int cells_wf_ctas_per_sm();
 // long pairs on a whole CTA (longpair.cu): one CTA per SM, kLongSlots boundary slots per CTA
 constexpr int kLongSlots = 8;
 constexpr int64_t kLongMinCols = 2048, kLongMinRows = 512;
 int long_pair_smem();
 cudaError_t launch_long_sw32(int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
                              int32_t* counter, cudaStream_t st);
+// alignment cells (cells.cu): long jobs (kLongMinCols, kLongMinRows) and the others; without
+// a.cell_units the long ones go to the kernel for scores of 2^28 and more (longpair.cu)
+cudaError_t launch_huge_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
+                              int32_t* counter, int32_t* res, cudaStream_t st);
 cudaError_t launch_long_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
                               int32_t* counter, int32_t* res, cudaStream_t st);
 cudaError_t launch_cells_wf(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,

@@ -22,7 +22,7 @@ struct DevBuf {
 enum BufId {
     B_DB, B_RAW, B_OFF, B_BLOCKS, B_TASKS, B_IDS, B_STREAM, B_SROW, B_OUT, B_OMAP, B_BND,
     B_FLAGS, B_PREF, B_FIRST, B_PAIRS, B_CELLS, B_SCRATCH, B_CHUNK, B_POUT, B_SOUT, B_MAT,
-    B_JOBS, B_RES, B_KEPT, B_KTOT, B_UNITS, B_RANGE, B_COUNT
+    B_JOBS, B_RES, B_KEPT, B_KTOT, B_UNITS, B_RANGE, B_BEST, B_COUNT
 };
 
 }  // namespace cm
@@ -48,7 +48,7 @@ struct cm_ctx {
     void* ranker = nullptr;                 // learned ranker state (ranker.cu)
     void (*ranker_free)(void*) = nullptr;
     int sw16_occ[3][33][4] = {};            // CTAs per SM by (W = 4/8/16, R, mode); 0 = unknown
-    int sw32_occ = 0, cells_occ = 0;        // ... of the int32 kernels
+    int sw32_occ = 0;                       // ... of the int32 rescoring kernel
 };
 
 namespace cm {

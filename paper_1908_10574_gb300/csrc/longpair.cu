@@ -176,7 +176,7 @@ cudaError_t launch_long_sw32(int grid, const SwArgs& a, const PairRef* pr, int32
     return cudaGetLastError();
 }
 
-cudaError_t launch_long_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
+cudaError_t launch_huge_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
                               int32_t* counter, int32_t* res, cudaStream_t st)
 {
     if (njobs == 0) return cudaSuccess;

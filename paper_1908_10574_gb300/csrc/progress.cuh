@@ -6,14 +6,15 @@
 #pragma once
 #include <cstdint>
 
+#include "cm_internal.h"
+
 namespace cm {
 namespace {
 
-constexpr int kPollLimit = 1 << 24;               // polls of ~100 ns before a wait gives up
-
-// waits (lane 0 polls) until `need` row groups are written; false on every lane once kPollLimit
+// waits (lane 0 polls) until `need` row groups are written; false on every lane once `limit`
 // polls have passed, or when another wait has given up and set `err`
-__device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, const int32_t* err)
+__device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, const int32_t* err,
+                                            int32_t limit = kPollLimit)
 {
     int ok = 1;
     if ((threadIdx.x & 31) == 0) {
@@ -21,7 +22,7 @@ __device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, c
             int32_t v;
             asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
             if (v >= need) break;
-            if (polls >= kPollLimit ||
+            if (polls >= limit ||
                 ((polls & 1023) == 1023 && *reinterpret_cast<const volatile int32_t*>(err) != 0)) {
                 ok = 0;
                 break;

@@ -1,5 +1,5 @@
-// Launchers of the Smith-Waterman kernels (templates in sw16_kernel.cuh): the int16x2
-// query-pair kernel by CTA width, the int32 rescoring kernel and the alignment-cells kernel.
+// Launchers of the Smith-Waterman kernels (templates in sw16_kernel.cuh); the int16x2
+// query-pair kernel by CTA width and the int32 rescoring kernel.
 #include "sw16_kernel.cuh"
 
 namespace cm {
@@ -70,36 +70,6 @@ cudaError_t launch_sw32(int R, int grid, const SwArgs& a, const PairRef* pr, int
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     sw32_kernel<16><<<grid, 32, smem, st>>>(a, pr, npairs, counter);
-    return cudaGetLastError();
-}
-
-}  // namespace cm
-
-namespace cm {
-
-int cells_wf_smem_bytes() { return kProfRows * 32 * lane_stride(8) * 4 + 32 * 8; }
-
-int cells_wf_ctas_per_sm()
-{
-    const int smem = cells_wf_smem_bytes();
-    if (cudaFuncSetAttribute(cells_wf_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) != cudaSuccess)
-        return 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cells_wf_kernel<8>, 32, smem) !=
-        cudaSuccess)
-        return 1;
-    return n;
-}
-
-cudaError_t launch_cells_wf(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
-                            int32_t* counter, int32_t* res, cudaStream_t st)
-{
-    const int smem = cells_wf_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(cells_wf_kernel<8>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    cells_wf_kernel<8><<<grid, 32, smem, st>>>(a, jobs, njobs, counter, res);
     return cudaGetLastError();
 }
 

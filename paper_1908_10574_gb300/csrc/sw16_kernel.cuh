@@ -420,74 +420,5 @@ __global__ void __launch_bounds__(32) sw32_kernel(const __grid_constant__ SwArgs
     }
 }
 
-// ---- alignment cells: score plus the first row-major cell reaching it, one warp per job ----
-// Rows stream the job's first sequence a[0..m) (reversed when J.reverse), columns hold its
-// second sequence b[0..n) (reversed likewise); cell scores are matrix[a residue][b residue].
-// The passes keep the largest score, then the smallest row, then the smallest column.
-template <int R>
-__global__ void __launch_bounds__(32) cells_wf_kernel(const __grid_constant__ SwArgs a,
-                                                     const CellJob* __restrict__ jobs,
-                                                     int32_t njobs, int32_t* counter,
-                                                     int32_t* __restrict__ res)
-{
-    using G = Geo<R>;
-    extern __shared__ __align__(16) uint8_t smem[];
-    int32_t* prof = reinterpret_cast<int32_t*>(smem);
-    uint8_t* qres = smem + (size_t)G::PROF_WORDS * 4;
-    __shared__ int16_t s_mat[kAlpha * kAlpha];
-    const int lane = threadIdx.x;
-    for (int i = lane; i < kAlpha * kAlpha; i += 32) s_mat[i] = a.mat[i];
-    __syncwarp();
-    const int o = a.gap_open, ge = a.gap_extend;
-    int2* bnd = reinterpret_cast<int2*>(a.bnd + (int64_t)blockIdx.x * a.bnd_stride);
-    auto no_wait = [](int32_t) { return true; };
-    auto no_publish = [](int32_t) {};
-
-    for (;;) {
-        int p = 0;
-        if (lane == 0) p = atomicAdd(counter, 1);
-        p = __shfl_sync(kFull, p, 0);
-        if (p >= njobs) break;
-        const CellJob J = jobs[p];
-        const uint8_t* ra = a.db + a.off[J.a];
-        const uint8_t* cb = a.db + a.off[J.b];
-        int64_t m = J.m;
-        const int64_t n = J.n;
-        const int npass = (n <= G::COLS) ? 1 : (int)((n + G::COLS - 1) / G::COLS);
-        if ((npass > 1 && m > a.bnd_stride) || m >= ((int64_t)1 << 30)) {
-            if (lane == 0) atomicExch(a.err, 1);
-            m = 0;
-        }
-        int32_t gbest = 0, grow = -1, gcol = -1;
-        for (int pass = 0; pass < npass && m > 0 && n > 0; ++pass) {
-            const int64_t c0 = (int64_t)pass * G::COLS;
-            __syncwarp();
-            for (int c = lane; c < G::COLS; c += 32) {
-                const int64_t cc = c0 + c;
-                qres[c] = (cc < n) ? (J.reverse ? cb[n - 1 - cc] : cb[cc]) : kPadCode;
-            }
-            __syncwarp();
-            for (int i = lane; i < kProfRows * G::COLS; i += 32) {
-                const int x = i / G::COLS, c = i - x * G::COLS;
-                const int ln = c / R, k = c - ln * R;
-                const int q = qres[c];
-                prof[x * G::ROWW + ln * G::LS + k] =
-                    (x != kPadCode && q != kPadCode) ? s_mat[x * kAlpha + q] + o : kSpad;
-            }
-            __syncwarp();
-            D32Best r;
-            dp32_pass<R, G::LS, true>(prof + lane * G::LS, ra, m, J.reverse != 0, o, ge,
-                                      pass > 0 ? bnd : nullptr, pass + 1 < npass ? bnd : nullptr,
-                                      (int32_t)c0 + lane * R, no_wait, no_publish, r);
-            if (first_max(r.b, r.r, r.c, gbest, grow, gcol)) { gbest = r.b; grow = r.r; gcol = r.c; }
-        }
-        if (lane == 0) {
-            res[3 * (int64_t)p] = gbest;
-            res[3 * (int64_t)p + 1] = gbest > 0 ? grow : -1;
-            res[3 * (int64_t)p + 2] = gbest > 0 ? gcol : -1;
-        }
-    }
-}
-
 }  // namespace
 }  // namespace cm
