@@ -20,14 +20,15 @@
 #include <cstring>
 
 #include "cm_internal.h"
+#include "wave32.cuh"
 
+namespace cm {
 namespace {
 
-constexpr int kNaThreads = 1024;                 // pairs in flight (one thread each)
-constexpr int kNaCols = 4096;                    // DP row length: second sequence <= 4095
-constexpr size_t kNaRowWords = 2ull * kNaThreads * kNaCols;   // H and F rows: 32 MiB
+constexpr int kNaWarps = 1024;                   // pairs in flight (one warp each)
+constexpr int kNaCols = 4096;                    // boundary row length: second sequence <= 4095
+constexpr size_t kNaRowWords = 2ull * kNaWarps * kNaCols;     // H and E rows: 32 MiB
 constexpr size_t kNaStatusWords = 64;            // status words after the rows
-constexpr int32_t kNaNeg = -(1 << 28);
 
 static __device__ __align__(256) int32_t g_na_scratch[kNaRowWords + kNaStatusWords];
 
@@ -44,86 +45,106 @@ void na_message(char* buf, int32_t len, const char* msg)
 }
 
 // status[0]: pair index out of range or bad offsets; status[1]: second sequence too long;
-// status[2]: residue code >= 20
+// status[2]: residue code >= 20.  One warp per pair.
 __global__ void na_check_kernel(const uint8_t* __restrict__ seqs, const int64_t* __restrict__ off,
                                 int32_t n_seqs, const int32_t* __restrict__ pairs, int64_t npairs,
                                 int32_t* status)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npairs;
-         p += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; p < npairs;
+         p += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int32_t x = pairs[2 * p], y = pairs[2 * p + 1];
         if (x < 0 || x >= n_seqs || y < 0 || y >= n_seqs) { atomicExch(status + 0, 1); continue; }
         const int64_t xb = off[x], xe = off[x + 1], yb = off[y], ye = off[y + 1];
         if (xb < 0 || xe < xb || yb < 0 || ye < yb) { atomicExch(status + 0, 1); continue; }
         if (ye - yb > kNaCols - 1) { atomicExch(status + 1, 1); continue; }
-        for (int64_t i = xb; i < xe; ++i)
-            if (seqs[i] >= 20) { atomicExch(status + 2, 1); break; }
-        for (int64_t i = yb; i < ye; ++i)
-            if (seqs[i] >= 20) { atomicExch(status + 2, 1); break; }
+        bool bad = false;
+        for (int64_t i = xb + lane; i < xe; i += 32) bad |= seqs[i] >= 20;
+        for (int64_t i = yb + lane; i < ye; i += 32) bad |= seqs[i] >= 20;
+        if (bad) atomicExch(status + 2, 1);
     }
 }
 
-__device__ int32_t na_gotoh(const uint8_t* a, int64_t m, const uint8_t* b, int64_t n, bool rev,
-                            const int16_t* mat, int32_t g1, int32_t ge, int32_t* H, int32_t* F,
-                            int32_t* bi, int32_t* bj)
+// Optimum of a[0..m) x b[0..n) (both back to front when `rev`) and its first row-major cell,
+// 1-based (0 when the score is 0).  wave32.cuh's wavefront with the rows held (strips of 256,
+// eight per lane) and the columns streamed: a strip hands its last row to the next through the
+// warp's boundary row, at most 4,095 pairs of words however long the first sequence is.
+__device__ int32_t na_optimum(const uint8_t* a, int64_t m, const uint8_t* b, int32_t n, bool rev,
+                              const int8_t* mat, int32_t g1, int32_t ge, uint2* prof, int2* bnd,
+                              int32_t* bi, int32_t* bj)
 {
-    for (int64_t j = 0; j <= n; ++j) { H[j * kNaThreads] = 0; F[j * kNaThreads] = kNaNeg; }
-    int32_t best = 0, ii = 0, jj = 0;
-    for (int64_t i = 1; i <= m; ++i) {
-        const int16_t* row = mat + (rev ? a[m - i] : a[i - 1]) * 20;
-        int32_t E = kNaNeg, hleft = 0, hdiag = 0;
-        for (int64_t j = 1; j <= n; ++j) {
-            const int32_t hup = H[j * kNaThreads];
-            E = max(E - ge, hleft - g1);
-            const int32_t f = max(F[j * kNaThreads] - ge, hup - g1);
-            F[j * kNaThreads] = f;
-            const int32_t h = max(max(hdiag + row[rev ? b[n - j] : b[j - 1]], 0), max(E, f));
-            hdiag = hup;
-            H[j * kNaThreads] = h;
-            hleft = h;
-            if (h > best) { best = h; ii = (int32_t)i; jj = (int32_t)j; }
-        }
+    constexpr int kRowsHeld = 32 * kWaveMaxR;
+    WaveStrip s;
+    s.prof = prof;
+    s.x = b;
+    s.xn = n;
+    s.reverse = rev;
+    s.o = g1;
+    s.ge = ge;
+    int32_t best = 0, row = -1, col = -1;
+    auto no_wait = [](int32_t) { return true; };
+    auto no_publish = [](int32_t) {};
+    for (int64_t i0 = 0; i0 < m && n > 0; i0 += kRowsHeld) {
+        s.bin = i0 > 0 ? bnd : nullptr;
+        s.bout = i0 + kRowsHeld < m ? bnd : nullptr;
+        s.y0 = (int32_t)i0;
+        __syncwarp();
+        wave_profile(prof, a, m, rev, i0, kWaveMaxR, mat, 20, 1, 20);
+        __syncwarp();
+        int32_t sc, x, y;
+        wave_strip<kWaveMaxR, true>(s, no_wait, no_publish, sc, x, y);
+        if (first_max(sc, y, x, best, row, col)) { best = sc; row = y; col = x; }
     }
-    *bi = ii;
-    *bj = jj;
+    *bi = row + 1;
+    *bj = col + 1;
     return best;
 }
 
-// one thread per pair; thread t keeps its H and F rows in columns t of the scratch rows
-__global__ void __launch_bounds__(128) na_cells_kernel(const uint8_t* __restrict__ seqs,
-                                                     const int64_t* __restrict__ off,
-                                                     const int32_t* __restrict__ pairs,
-                                                     int64_t npairs, const NaMatrix mat_in,
-                                                     int32_t g1, int32_t ge,
-                                                     int32_t* __restrict__ cells,
-                                                     int32_t* scratch)
+// One warp per pair, pairs taken from a queue.  Bound by the serial chain of the longest pairs;
+// 200 pairs of up to 600 residues: 0.58 ms per call, 252 ms with one thread per pair and its
+// rows in the scratch array.
+__global__ void __launch_bounds__(32) na_cells_kernel(const uint8_t* __restrict__ seqs,
+                                                      const int64_t* __restrict__ off,
+                                                      const int32_t* __restrict__ pairs,
+                                                      int64_t npairs, const NaMatrix mat_in,
+                                                      int32_t g1, int32_t ge,
+                                                      int32_t* __restrict__ cells,
+                                                      int32_t* scratch, int32_t* ticket)
 {
-    __shared__ int16_t mat[400];
-    for (int i = threadIdx.x; i < 400; i += blockDim.x) mat[i] = mat_in.v[i];
-    __syncthreads();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= kNaThreads) return;
-    int32_t* H = scratch + t;
-    int32_t* F = scratch + (size_t)kNaThreads * kNaCols + t;
-    for (int64_t p = t; p < npairs; p += kNaThreads) {
-        const int32_t x = pairs[2 * p], y = pairs[2 * p + 1];
+    __shared__ int8_t mat[400];
+    __shared__ uint2 prof[kWaveProf];
+    const int lane = threadIdx.x;
+    for (int i = lane; i < 400; i += 32) mat[i] = (int8_t)mat_in.v[i];
+    __syncwarp();
+    int2* bnd = reinterpret_cast<int2*>(scratch) + (size_t)blockIdx.x * kNaCols;
+    for (;;) {
+        uint32_t p = 0;
+        if (lane == 0) p = (uint32_t)atomicAdd(ticket, 1);
+        p = __shfl_sync(0xffffffffu, p, 0);
+        if (p >= npairs) break;
+        const int32_t x = pairs[2 * (int64_t)p], y = pairs[2 * (int64_t)p + 1];
         const uint8_t* a = seqs + off[x];
         const uint8_t* b = seqs + off[y];
-        const int64_t m = off[x + 1] - off[x], n = off[y + 1] - off[y];
-        int32_t* c = cells + 5 * p;
-        int32_t ie, je, ri, rj;
-        const int32_t best = na_gotoh(a, m, b, n, false, mat, g1, ge, H, F, &ie, &je);
-        c[0] = best;
-        if (best == 0) { c[1] = c[2] = c[3] = c[4] = 0; continue; }
-        na_gotoh(a, ie, b, je, true, mat, g1, ge, H, F, &ri, &rj);
-        c[1] = ie - ri + 1;
-        c[2] = ie;
-        c[3] = je - rj + 1;
-        c[4] = je;
+        const int64_t m = off[x + 1] - off[x];
+        const int32_t n = (int32_t)(off[y + 1] - off[y]);
+        int32_t ie, je, ri = 0, rj = 0;
+        const int32_t best = na_optimum(a, m, b, n, false, mat, g1, ge, prof, bnd, &ie, &je);
+        if (best > 0) na_optimum(a, ie, b, je, true, mat, g1, ge, prof, bnd, &ri, &rj);
+        if (lane == 0) {
+            int32_t* c = cells + 5 * (int64_t)p;
+            c[0] = best;
+            c[1] = best > 0 ? ie - ri + 1 : 0;
+            c[2] = best > 0 ? ie : 0;
+            c[3] = best > 0 ? je - rj + 1 : 0;
+            c[4] = best > 0 ? je : 0;
+        }
     }
 }
 
 }  // namespace
+}  // namespace cm
+
+using namespace cm;
 
 extern "C" int sw_cells_batch_noalloc(const uint8_t* seqs, const int64_t* offsets,
                                       int32_t n_seqs, const int32_t* pairs, int64_t n_pairs,
@@ -175,7 +196,7 @@ extern "C" int sw_cells_batch_noalloc(const uint8_t* seqs, const int64_t* offset
 
     cudaError_t e = cudaMemsetAsync(status, 0, kNaStatusWords * sizeof(int32_t), st);
     if (e == cudaSuccess) {
-        const int64_t blocks = std::min<int64_t>((n_pairs + 255) / 256, 4096);
+        const int64_t blocks = std::min<int64_t>((n_pairs + 7) / 8, 4096);
         na_check_kernel<<<(unsigned)blocks, 256, 0, st>>>(seqs, offsets, n_seqs, pairs, n_pairs,
                                                            status);
         e = cudaGetLastError();
@@ -200,9 +221,8 @@ extern "C" int sw_cells_batch_noalloc(const uint8_t* seqs, const int64_t* offset
         na_message(err_msg, err_len, "residue code >= 20 in a paired sequence");
         return CM_ERR_RESIDUE;
     }
-    na_cells_kernel<<<kNaThreads / 128, 128, 0, st>>>(seqs, offsets, pairs, n_pairs, M,
-                                                      (int32_t)g1, gap_extend, cells_out,
-                                                      scratch);
+    na_cells_kernel<<<(unsigned)std::min<int64_t>(n_pairs, kNaWarps), 32, 0, st>>>(
+        seqs, offsets, pairs, n_pairs, M, (int32_t)g1, gap_extend, cells_out, scratch, status + 8);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
