@@ -233,8 +233,10 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
 
     // Launches.  All single-query tasks run in one launch, each CTA a contiguous range of them
     // of an equal share of the cost: first the tasks of several passes, then tile by tile (the
-    // plan's order).  The query pairs run in one persistent launch per (register tile, mode)
-    // bin.  (Builds without the single-query launcher give its tasks a launch per bin too.)
+    // plan's order).  The query pairs of a plan that does not fill the chip tile by tile run in
+    // one launch too (with 16-warp CTAs, one per SM); those of a large plan, or of narrower CTAs,
+    // in a persistent launch per (register tile, mode) bin.  (Builds without the launchers of
+    // several tiles get a launch per bin.)
     struct Launch {
         int R, mode, grid, warps_per_cta;
         size_t i0, i1;
@@ -306,18 +308,33 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
             const int warps = (int)std::min<int64_t>(kSingleWarps, (nu + grid - 1) / grid);
             launches.push_back({0, kModeTwo, grid, warps, 0, n_single, true, 0});
             // the plan's remaining tasks, in its order
-            std::vector<SwTask> t2;
-            std::vector<int> r2;
+            size_t k = 0;
             for (size_t i = 0; i < plan.tasks.size(); ++i)
                 if (!single(plan.tasks[i])) {
-                    t2.push_back(plan.tasks[i]);
-                    r2.push_back(plan.task_R[i]);
+                    plan.tasks[k] = plan.tasks[i];
+                    plan.task_R[k] = plan.task_R[i];
+                    plan.keys[k++] = plan.keys[i];
                 }
-            plan.tasks.swap(t2);
-            plan.task_R.swap(r2);
+            plan.tasks.resize(k);
+            plan.task_R.resize(k);
+            plan.keys.resize(k);
         }
     }
-    for (size_t i0 = 0; i0 < plan.tasks.size();) {
+    int pair_smem = 0;
+    const bool one_pairs = W == 16 && launch_sw16_pairs && !plan.tasks.empty() &&
+                           (int64_t)plan.tasks.size() <= (int64_t)kMergedTasks * c->num_sms;
+    if (one_pairs) {                              // longest first, whatever their tile
+        const size_t n = plan.tasks.size();
+        std::vector<std::pair<int64_t, size_t>> order(n);
+        for (size_t i = 0; i < n; ++i) order[i] = {-plan.keys[i].first, i};
+        std::sort(order.begin(), order.end());
+        std::vector<SwTask> t2(n);
+        for (size_t i = 0; i < n; ++i) t2[i] = plan.tasks[order[i].second];
+        plan.tasks.swap(t2);
+        for (const SwTask& t : plan.tasks) pair_smem = std::max(pair_smem, sw16_pair_smem(t.R, t.mode));
+        launches.push_back({0, kModePair, (int)std::min<int64_t>((int64_t)n, c->num_sms), W, 0, n, false, 0});
+    }
+    for (size_t i0 = one_pairs ? plan.tasks.size() : 0; i0 < plan.tasks.size();) {
         const int key = plan.task_R[i0];
         size_t i1 = i0;
         while (i1 < plan.tasks.size() && plan.task_R[i1] == key) ++i1;
@@ -370,8 +387,9 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         a.progress = L.single ? d_tickets + L.grid : nullptr;
         a.piped = d_bnd;
         const cudaStream_t ls = side ? c->aux : st;
-        le = L.single ? launch_sw16_single(L.grid, L.warps_per_cta, a, ls)
-                      : launch_sw16(L.R, W, L.mode, L.grid, a, ls);
+        le = L.single    ? launch_sw16_single(L.grid, L.warps_per_cta, a, ls)
+             : one_pairs ? launch_sw16_pairs(W, L.grid, pair_smem, a, ls)
+                         : launch_sw16(L.R, W, L.mode, L.grid, a, ls);
         c->stats.launches += 1;
         c->stats.sw16_launches += 1;
     }

@@ -179,9 +179,25 @@ struct KeptList {
     int64_t rowbase;        // first stream row of the list
 };
 
-// ---- launchers (sw16.cu) ---------------------------------------------------------------
+// ---- launchers (sw16.cu, sw16_pair.cu, sw16_single.cu) ---------------------------------
+// Words per lane in a profile row of the query-pair kernel: R rounded up to a multiple of 4
+// (16-byte loads), plus 4 more when that is an even number of 16-byte units, so that the eight
+// lanes of a quarter warp always read eight distinct 16-byte bank groups whatever residues they
+// look up.
+inline __host__ __device__ constexpr int lane_stride(int R)
+{
+    return (((R + 3) / 4) & 1) ? (R + 3) / 4 * 4 : (R + 3) / 4 * 4 + 4;
+}
+// shared memory of a query-pair CTA: the profile of one tile
+inline constexpr int sw16_pair_smem(int R, int mode)
+{
+    return kProfRows * (mode == kModeSeg16 ? 16 : 32) * lane_stride(R) * 4;
+}
 int sw16_ctas_per_sm(int R, int W, int mode);
+// query pairs: the tasks of one tile and mode, or (weak, see launch_sw16_single) of all of them
 cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st);
+cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaStream_t st)
+    __attribute__((weak));
 // Every single-query task (kModeTwo, kModeTwo16; any tile width) in one launch of `grid` CTAs of
 // `warps` warps, a unit per warp at a time; CTA b owns the units [ranges[b], ranges[b + 1]),
 // task_counter[b] is its ticket.  Slots of bnd_stride rows for the units of all passes are

@@ -97,6 +97,7 @@ int ensure(cm_ctx* c, BufId id, size_t count, T** out)
 // the long queries of a larger plan, which fill the chip by their number, run their passes
 // one after another
 constexpr int64_t kPipedRows = (int64_t)1 << 26;
+constexpr int kMergedTasks = 64;   // query-pair tasks per SM up to which one launch takes all tiles
 constexpr int kTaskBins = 32 * 4;
 constexpr int kFlagWords = 8 + kTaskBins;
 

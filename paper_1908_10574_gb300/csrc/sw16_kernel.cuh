@@ -35,14 +35,6 @@ namespace {
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kSpad = -1024;   // profile entry of pad rows / pad columns (any value <= 0 works)
 
-// Words per lane in a profile row: R rounded up to a multiple of 4 (16-byte loads), plus 4
-// more when that is an even number of 16-byte units, so that the eight lanes of a quarter
-// warp always read eight distinct 16-byte bank groups whatever residues they look up.
-__host__ __device__ constexpr int lane_stride(int R)
-{
-    return (((R + 3) / 4) & 1) ? (R + 3) / 4 * 4 : (R + 3) / 4 * 4 + 4;
-}
-
 // Tile geometry: SEG lanes (32, or 16 for a half-warp segment) of R columns each.
 template <int R, int SEG = 32>
 struct Geo {
