@@ -11,10 +11,6 @@
 #include "batches.h"
 #include "ctx.h"
 
-namespace cm {
-int sw32_ctas_per_sm();
-}  // namespace cm
-
 using namespace cm;
 
 namespace cm {
@@ -178,6 +174,113 @@ int64_t longest_stream(const int64_t* srow, int32_t s0, int32_t s1, int n)
         prev = s;
     }
     return longest;
+}
+
+}  // namespace
+
+namespace {
+
+// The int32 passes over a list of nj pairs, nlong long ones first (strips.cu): rows(i) and
+// cols(i) of pair i; launch(lng, a, j0, count, ticket, stream) launches pairs [j0, j0 + count).
+// In rounds whose boundary columns hold at most kPipedRows rows; a round's long pairs run on the
+// auxiliary stream beside its other ones, so the few warps of their pipelines do not have the
+// chip to themselves.  With max_score > 0 (cells), a round whose long pairs may score 2^28 runs
+// them on the kernel for such scores.
+template <class Rows, class Cols, class Launch>
+int run_strips(cm_ctx* c, const Prepared& P, SwArgs a, int32_t nj, int32_t nlong, int32_t max_score,
+               Rows&& rows_of, Cols&& cols_of, Launch&& launch)
+{
+    const cudaStream_t st = c->stream;
+    a.num_sms = c->num_sms;
+    a.bnd_stride = P.maxlen + 64;
+    for (int32_t q = 0; q < nj;) {
+        std::vector<CellUnit> units;
+        int64_t rows = 0, long_units = 0;
+        bool huge = false;
+        int32_t e = q;
+        for (; e < nj; ++e) {
+            const int64_t m = rows_of(e), n = cols_of(e);
+            const int32_t strips = cell_strips(m, n), first = e < nlong ? q : std::max(q, nlong);
+            const int64_t more = strips > 1 ? stream_rows(m) : 0;      // whole row groups
+            if (e > q && (rows + more > kPipedRows || (int64_t)units.size() + strips > INT32_MAX)) break;
+            huge = huge || std::min(m, n) * max_score >= kWaveScoreLimit;
+            for (int32_t t = 0; t < strips; ++t)
+                units.push_back({e - first, t, e < nlong ? c->wait_limit : kPollLimit, 0, rows});
+            rows += more;
+            if (e < nlong) long_units = (int64_t)units.size();
+        }
+        int r;
+        const int64_t nu = (int64_t)units.size();
+        CellUnit* d_units;
+        int4* d_best;
+        uint2* d_bnd;
+        int32_t* d_prog;
+        ENSURE(B_PROG, kProgWords + nu, d_prog);
+        ENSURE(B_UNITS, nu, d_units);
+        ENSURE(B_BEST, nu, d_best);
+        const int32_t lend = std::min(std::max(q, nlong), e);          // [q, lend) long, [lend, e) not
+        const int64_t huge_rows =
+            huge ? std::min<int64_t>(std::max(lend - q, 1), c->num_sms) * kLongSlots * a.bnd_stride : 0;
+        ENSURE(B_BND, rows + huge_rows, d_bnd);
+        if ((r = copy_in(c, d_units, units.data(), units.size() * sizeof(CellUnit), false))) return r;
+        CUDA_TRY(cudaMemsetAsync(d_prog, 0, (kProgWords + nu) * sizeof(int32_t), st));
+        a.err = d_prog;
+        auto part = [&](int32_t j0, int32_t j1, int64_t u0, int64_t u1, bool lng) {
+            const bool hg = lng && huge;
+            a.bnd = d_bnd + (hg ? rows : 0);
+            a.cell_units = hg ? nullptr : d_units + u0;
+            a.ncells = (int32_t)(u1 - u0);
+            a.progress = d_prog + kProgWords + u0;
+            a.cell_best = d_best + u0;
+            c->stats.launches += 1;
+            return launch(lng, a, j0, j1 - j0, d_prog + (lng ? 1 : 2), lng ? c->aux : st);
+        };
+        cudaError_t le = cudaSuccess;
+        if (lend > q) {
+            CUDA_TRY(cudaEventRecord(c->fork, st));
+            CUDA_TRY(cudaStreamWaitEvent(c->aux, c->fork, 0));
+            le = part(q, lend, 0, long_units, true);
+        }
+        if (e > lend && le == cudaSuccess) le = part(lend, e, long_units, nu, false);
+        if (lend > q) {                           // no launch of this call outlives it
+            CUDA_TRY(cudaEventRecord(c->join, c->aux));
+            CUDA_TRY(cudaStreamWaitEvent(st, c->join, 0));
+        }
+        CUDA_TRY(le);
+        int32_t kerr = 0;
+        CUDA_TRY(cudaMemcpyAsync(&kerr, d_prog, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(cudaStreamSynchronize(st));
+        if (kerr == 2) return fail(c, CM_ERR_TIMEOUT, "a long-pair pipeline wait gave up");
+        if (kerr) return fail(c, CM_ERR_INTERNAL, "an int32 kernel's bounds check fired");
+        q = e;
+    }
+    return CM_OK;
+}
+
+// int32 scores of a list of pairs on the device (lst also holds it), into their slots of a.out
+int rescore(cm_ctx* c, const Prepared& P, const SwArgs& a, std::vector<PairRef>& lst, PairRef* d_pref)
+{
+    // long pairs first, then the rest, each longest first (the warps take units in order)
+    auto is_long = [&](const PairRef& x) {
+        return P.len(x.q) >= kLongMinCols && P.len(x.x) >= kLongMinRows;
+    };
+    std::stable_sort(lst.begin(), lst.end(), [&](const PairRef& x, const PairRef& y) {
+        const bool lx = is_long(x), ly = is_long(y);
+        if (lx != ly) return lx;
+        return P.len(x.q) * P.len(x.x) > P.len(y.q) * P.len(y.x);
+    });
+    const int32_t n = (int32_t)lst.size();
+    int32_t nlong = 0;
+    while (nlong < n && is_long(lst[nlong])) ++nlong;
+    const int r = copy_in(c, d_pref, lst.data(), lst.size() * sizeof(PairRef), false);
+    if (r) return r;
+    return run_strips(
+        c, P, a, n, nlong, 0, [&](int32_t i) { return P.len(lst[i].x); },
+        [&](int32_t i) { return P.len(lst[i].q); },
+        [&](bool lng, const SwArgs& u, int32_t j0, int32_t count, int32_t* ticket, cudaStream_t s) {
+            return lng ? launch_long_sw32(std::min(count, c->num_sms), u, d_pref + j0, count, ticket, s)
+                       : launch_sw32(kWaveMaxR, std::min(count, c->num_sms), u, d_pref + j0, count, ticket, s);
+        });
 }
 
 }  // namespace
@@ -414,35 +517,10 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         if (cnt == 0) break;
         const int32_t n = std::min(cnt, cap);
         c->stats.saturated += n;
-        // Long pairs (many column passes) first, on whole CTAs; the rest longest first on one
-        // warp each (the persistent warps claim them in order).
         std::vector<PairRef> lst((size_t)n);
         CUDA_TRY(cudaMemcpyAsync(lst.data(), d_pref, n * sizeof(PairRef), cudaMemcpyDeviceToHost, st));
         CUDA_TRY(cudaStreamSynchronize(st));
-        auto is_long = [&](const PairRef& x) {
-            return P.len(x.q) >= kLongMinCols && P.len(x.x) >= kLongMinRows;
-        };
-        std::stable_sort(lst.begin(), lst.end(), [&](const PairRef& x, const PairRef& y) {
-            const bool lx = is_long(x), ly = is_long(y);
-            if (lx != ly) return lx;
-            return P.len(x.q) * P.len(x.x) > P.len(y.q) * P.len(y.x);
-        });
-        if ((r = copy_in(c, d_pref, lst.data(), lst.size() * sizeof(PairRef), false))) return r;
-        int32_t nlong = 0;
-        while (nlong < n && is_long(lst[nlong])) ++nlong;
-        if (c->sw32_occ == 0) c->sw32_occ = std::max(1, sw32_ctas_per_sm());
-        const int64_t grid32 = std::min<int64_t>(n - nlong, (int64_t)c->num_sms * c->sw32_occ);
-        const int64_t grid_long = std::min<int64_t>(nlong, c->num_sms);
-        ENSURE(B_BND, std::max(grid32, grid_long * kLongSlots) * stride, d_bnd);
-        a.bnd = d_bnd;
-        if (nlong > 0) {
-            CUDA_TRY(launch_long_sw32((int)grid_long, a, d_pref, nlong, d_flags + 5, st));
-            c->stats.launches += 1;
-        }
-        if (n > nlong) {
-            CUDA_TRY(launch_sw32(16, (int)grid32, a, d_pref + nlong, n - nlong, d_flags + 3, st));
-            c->stats.launches += 1;
-        }
+        if ((r = rescore(c, P, a, lst, d_pref))) return r;
         // every full round rescored `cap` distinct slots (a rescored slot no longer holds the
         // saturation mark), so more rounds than slots / cap means no progress
         if ((int64_t)round * cap > plan.nslots)
@@ -674,58 +752,21 @@ int score_pairs_int32(cm_ctx* c, const Prepared& P, const std::vector<int32_t>& 
     const cudaStream_t st = c->stream;
     std::vector<PairRef> lst((size_t)n);
     for (int64_t k = 0; k < n; ++k) lst[k] = PairRef{pairs[2 * k], pairs[2 * k + 1], 0, 0, k};
-    // long pairs first, for whole CTAs; the rest longest first on one warp each
-    auto is_long = [&](const PairRef& x) {
-        return P.len(x.q) >= kLongMinCols && P.len(x.x) >= kLongMinRows;
-    };
-    std::stable_sort(lst.begin(), lst.end(), [&](const PairRef& x, const PairRef& y) {
-        const bool lx = is_long(x), ly = is_long(y);
-        if (lx != ly) return lx;
-        return P.len(x.q) * P.len(x.x) > P.len(y.q) * P.len(y.x);
-    });
-    int32_t nlong = 0;
-    while (nlong < n && is_long(lst[nlong])) ++nlong;
     PairRef* d_pref;
-    int32_t *d_out, *d_flags;
-    uint2* d_bnd;
+    int32_t* d_out;
     ENSURE(B_PREF, n, d_pref);
     ENSURE(B_OUT, n, d_out);
-    ENSURE(B_FLAGS, kFlagWords, d_flags);
-    const int64_t stride = (P.maxlen + 64 + 1) & ~(int64_t)1;
-    if (c->sw32_occ == 0) c->sw32_occ = std::max(1, sw32_ctas_per_sm());
-    const int64_t grid32 = std::min<int64_t>(n - nlong, (int64_t)c->num_sms * c->sw32_occ);
-    const int64_t grid_long = std::min<int64_t>(nlong, c->num_sms);
-    ENSURE(B_BND, std::max(grid32, grid_long * kLongSlots) * stride, d_bnd);
-    int r = copy_in(c, d_pref, lst.data(), lst.size() * sizeof(PairRef), false);
-    if (r) return r;
-    CUDA_TRY(cudaMemsetAsync(d_flags, 0, kFlagWords * sizeof(int32_t), st));
     SwArgs a{};
     a.db = P.db;
     a.off = P.off;
     a.out = d_out;
-    a.err = d_flags + 1;
-    a.wait_limit = c->wait_limit;
     std::memcpy(a.mat, P.mat, sizeof(a.mat));
     a.gap_open = P.g1;
     a.gap_extend = P.ge;
-    a.beta = P.beta;
-    a.sat_thr = P.sat_thr;
-    a.bnd = d_bnd;
-    a.bnd_stride = stride;
-    if (nlong > 0) {
-        CUDA_TRY(launch_long_sw32((int)grid_long, a, d_pref, nlong, d_flags + 5, st));
-        c->stats.launches += 1;
-    }
-    if (n > nlong) {
-        CUDA_TRY(launch_sw32(16, (int)grid32, a, d_pref + nlong, (int32_t)(n - nlong), d_flags + 3, st));
-        c->stats.launches += 1;
-    }
-    int32_t kerr = 0;
+    const int r = rescore(c, P, a, lst, d_pref);
+    if (r) return r;
     CUDA_TRY(cudaMemcpyAsync(scores.data(), d_out, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaMemcpyAsync(&kerr, d_flags + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    if (kerr == 2) return fail(c, CM_ERR_TIMEOUT, "a long-pair pipeline wait gave up");
-    if (kerr) return fail(c, CM_ERR_INTERNAL, "kernel bounds check fired (boundary buffer)");
     c->stats.pairs += n;
     return CM_OK;
 }
@@ -755,7 +796,7 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
     int32_t max_score = 0;
     for (int i = 0; i < kAlpha * kAlpha; ++i) max_score = std::max<int32_t>(max_score, P.mat[i]);
     CellJob* d_jobs;
-    int32_t *d_res, *d_flags;
+    int32_t* d_res;
     ENSURE(B_JOBS, n_pairs, d_jobs);
     ENSURE(B_RES, 3 * n_pairs, d_res);
     SwArgs a{};
@@ -765,85 +806,22 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
     std::memcpy(a.mat, P.mat, sizeof(a.mat));
     a.gap_open = P.g1;
     a.gap_extend = P.ge;
-    a.num_sms = c->num_sms;
-    // All jobs (nlong long ones first), in rounds whose boundary columns hold at most kPipedRows
-    // rows; a round's long jobs run on the auxiliary stream beside its other ones, so the few
-    // warps of their pipelines do not have the chip to themselves.
-    auto run_jobs = [&](int32_t nlong) -> int {
-        const int32_t nj = (int32_t)jobs.size();
-        for (int32_t q = 0; q < nj;) {
-            std::vector<CellUnit> units;
-            int64_t rows = 0, ulong_ = 0;
-            bool huge = false;
-            int32_t e = q;
-            for (; e < nj; ++e) {
-                const CellJob& J = jobs[e];
-                const int32_t strips = cell_strips(J.m, J.n), first = e < nlong ? q : std::max(q, nlong);
-                const int64_t more = strips > 1 ? stream_rows(J.m) : 0;   // whole row groups
-                if (e > q && (rows + more > kPipedRows || (int64_t)units.size() + strips > INT32_MAX)) break;
-                huge = huge || std::min<int64_t>(J.m, J.n) * max_score >= kWaveScoreLimit;
-                for (int32_t t = 0; t < strips; ++t)
-                    units.push_back({e - first, t, e < nlong ? c->wait_limit : kPollLimit, 0, rows});
-                rows += more;
-                if (e < nlong) ulong_ = (int64_t)units.size();
-            }
-            int r;
-            const int64_t nu = (int64_t)units.size();
-            CellUnit* d_units;
-            int4* d_best;
-            uint2* d_bnd;
-            ENSURE(B_FLAGS, kFlagWords + nu, d_flags);
-            ENSURE(B_UNITS, nu, d_units);
-            ENSURE(B_BEST, nu, d_best);
-            const int32_t lend = std::min(std::max(q, nlong), e);      // [q, lend) long, [lend, e) not
-            const int huge_grid = (int)std::min<int64_t>(std::max(lend - q, 1), c->num_sms);
-            const int64_t huge_rows = huge ? (int64_t)huge_grid * kLongSlots * (P.maxlen + 64) : 0;
-            ENSURE(B_BND, rows + huge_rows, d_bnd);
-            if ((r = copy_in(c, d_units, units.data(), units.size() * sizeof(CellUnit), false))) return r;
-            CUDA_TRY(cudaMemsetAsync(d_flags, 0, (kFlagWords + nu) * sizeof(int32_t), st));
-            a.err = d_flags + 1;
-            auto part = [&](int32_t j0, int32_t j1, int64_t u0, int64_t u1, bool lng) {
-                const bool hg = lng && huge;
-                a.bnd = d_bnd + (hg ? rows : 0);
-                a.bnd_stride = P.maxlen + 64;
-                a.cell_units = hg ? nullptr : d_units + u0;
-                a.ncells = (int32_t)(u1 - u0);
-                a.progress = d_flags + kFlagWords + u0;
-                a.cell_best = d_best + u0;
-                int32_t* out = d_res + 3 * (int64_t)j0;
-                c->stats.launches += 1;
-                return lng ? launch_long_cells(huge_grid, a, d_jobs + j0, j1 - j0, d_flags + 6, out, c->aux)
-                           : launch_cells_wf((int)std::min<int64_t>(j1 - j0, c->num_sms), a, d_jobs + j0,
-                                             j1 - j0, d_flags + 4, out, st);
-            };
-            cudaError_t le = cudaSuccess;
-            if (lend > q) {
-                CUDA_TRY(cudaEventRecord(c->fork, st));
-                CUDA_TRY(cudaStreamWaitEvent(c->aux, c->fork, 0));
-                le = part(q, lend, 0, ulong_, true);
-            }
-            if (e > lend && le == cudaSuccess) le = part(lend, e, ulong_, nu, false);
-            if (lend > q) {                       // no launch of this call outlives it
-                CUDA_TRY(cudaEventRecord(c->join, c->aux));
-                CUDA_TRY(cudaStreamWaitEvent(st, c->join, 0));
-            }
-            CUDA_TRY(le);
-            int32_t kerr = 0;
-            CUDA_TRY(cudaMemcpyAsync(&kerr, a.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-            CUDA_TRY(cudaStreamSynchronize(st));
-            if (kerr == 2) return fail(c, CM_ERR_TIMEOUT, "a long-pair pipeline wait gave up");
-            if (kerr) return fail(c, CM_ERR_INTERNAL, "cells kernel bounds check fired");
-            q = e;
-        }
-        return CM_OK;
-    };
     std::vector<int32_t> fwd((size_t)n_pairs * 3);
     for (int dir = 0; dir < 2; ++dir) {
         int r = copy_in(c, d_jobs, jobs.data(), jobs.size() * sizeof(CellJob), false);
         if (r) return r;
         int32_t nlong = 0;
         while (nlong < (int32_t)jobs.size() && is_long(jobs[nlong])) ++nlong;
-        if ((r = run_jobs(nlong))) return r;
+        r = run_strips(
+            c, P, a, (int32_t)jobs.size(), nlong, max_score, [&](int32_t i) { return (int64_t)jobs[i].m; },
+            [&](int32_t i) { return (int64_t)jobs[i].n; },
+            [&](bool lng, const SwArgs& u, int32_t j0, int32_t count, int32_t* ticket, cudaStream_t s) {
+                int32_t* res = d_res + 3 * (int64_t)j0;
+                const int grid = std::min(count, c->num_sms);
+                return lng ? launch_long_cells(grid, u, d_jobs + j0, count, ticket, res, s)
+                           : launch_cells_wf(grid, u, d_jobs + j0, count, ticket, res, s);
+            });
+        if (r) return r;
         std::vector<int32_t> res(jobs.size() * 3);
         CUDA_TRY(cudaMemcpyAsync(res.data(), d_res, res.size() * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, st));

@@ -104,10 +104,10 @@ struct SwArgs {
     const int32_t* ranges;      // ... first unit of each CTA (grid + 1)
     int32_t* progress;          // ... boundary row groups written by each unit (zeroed)
     uint2* piped;               // ... boundary columns of the pipelined units
-    const CellUnit* cell_units; // alignment-cells launch: its units (null: the huge-score kernel)
+    const CellUnit* cell_units; // int32 launch: its units (null: the huge-score kernel)
     int32_t ncells;
     int32_t num_sms;
-    int4* cell_best;            // ... best cell up to each unit's strip
+    int4* cell_best;            // ... best so far up to each unit's strip
     const int32_t* ids;         // id pool
     const uint8_t* streams;     // stream pool
     const int64_t* srows;       // row pool
@@ -143,8 +143,8 @@ struct CellJob {
     int32_t pad;
 };
 
-// Strips of the alignment-cells wavefront (wave32.cuh): at most 32 lanes x kWaveMaxR columns of
-// b, of equal width; a unit of its launch is one strip of one job.
+// Strips of the int32 wavefront (wave32.cuh): at most 32 lanes x kWaveMaxR columns, of equal
+// width; a unit of its launches (strips.cu) is one strip of one job.
 constexpr int kWaveMaxR = 8;           // columns per lane: two profile words
 constexpr int64_t kWaveScoreLimit = (int64_t)1 << 28;
 constexpr int32_t kPollLimit = 1 << 24;   // polls of ~100 ns before a device wait gives up
@@ -208,21 +208,21 @@ cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_
     __attribute__((weak));
 cudaError_t launch_sw32(int R, int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
                         int32_t* counter, cudaStream_t st);
-int sw32_smem_bytes(int R);
-// long pairs on a whole CTA (longpair.cu): one CTA per SM, kLongSlots boundary slots per CTA
-constexpr int kLongSlots = 8;
+// int32 passes over lists of pairs (strips.cu): a.cell_units, a.ncells, a.progress, a.cell_best
+// hold the list's units.  Long pairs (kLongMinCols, kLongMinRows) have launches of their own,
+// whose waits cm_set_wait_limit bounds.
 constexpr int64_t kLongMinCols = 2048, kLongMinRows = 512;
-int long_pair_smem();
 cudaError_t launch_long_sw32(int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
                              int32_t* counter, cudaStream_t st);
-// alignment cells (cells.cu): long jobs (kLongMinCols, kLongMinRows) and the others; without
-// a.cell_units the long ones go to the kernel for scores of 2^28 and more (longpair.cu)
-cudaError_t launch_huge_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
-                              int32_t* counter, int32_t* res, cudaStream_t st);
 cudaError_t launch_long_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
                               int32_t* counter, int32_t* res, cudaStream_t st);
 cudaError_t launch_cells_wf(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
                             int32_t* counter, int32_t* res, cudaStream_t st);
+// alignment cells where scores may reach 2^28 (longpair.cu; launch_long_cells without
+// a.cell_units): kLongSlots boundary slots of bnd_stride rows per CTA
+constexpr int kLongSlots = 8;
+cudaError_t launch_huge_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t njobs,
+                              int32_t* counter, int32_t* res, cudaStream_t st);
 
 // ---- pack.cu ---------------------------------------------------------------------------
 // letters of the 20-letter alphabet (alpha 20) or also B, Z, X, * (alpha 24) -> codes

@@ -22,7 +22,7 @@ struct DevBuf {
 enum BufId {
     B_DB, B_RAW, B_OFF, B_BLOCKS, B_TASKS, B_IDS, B_STREAM, B_SROW, B_OUT, B_OMAP, B_BND,
     B_FLAGS, B_PREF, B_FIRST, B_PAIRS, B_CELLS, B_SCRATCH, B_CHUNK, B_POUT, B_SOUT, B_MAT,
-    B_JOBS, B_RES, B_KEPT, B_KTOT, B_UNITS, B_RANGE, B_BEST, B_COUNT
+    B_JOBS, B_RES, B_KEPT, B_KTOT, B_UNITS, B_RANGE, B_BEST, B_PROG, B_COUNT
 };
 
 }  // namespace cm
@@ -48,7 +48,6 @@ struct cm_ctx {
     void* ranker = nullptr;                 // learned ranker state (ranker.cu)
     void (*ranker_free)(void*) = nullptr;
     int sw16_occ[3][33][4] = {};            // CTAs per SM by (W = 4/8/16, R, mode); 0 = unknown
-    int sw32_occ = 0;                       // ... of the int32 rescoring kernel
 };
 
 namespace cm {
@@ -90,9 +89,10 @@ int ensure(cm_ctx* c, BufId id, size_t count, T** out)
     return r;
 }
 
-// B_FLAGS layout (int32 words): [1] kernel bounds-check flag, [2..3] int32-rerun list count and
-// ticket, [4..7] other kernels' tickets, [8 ..) one task ticket per (tile width, launch mode)
-// bin of the int16x2 kernel.
+// B_FLAGS layout (int32 words): [1] kernel bounds-check flag, [2] int32-rerun list count,
+// [8 ..) one task ticket per launch of the int16x2 kernels.  B_PROG, of the int32 passes: [0]
+// error flag, [1..2] tickets of the long and the other pairs, [kProgWords ..) progress words.
+constexpr int kProgWords = 4;
 // rows of boundary columns kept for pipelined column passes (8 bytes each: 512 MB at most);
 // the long queries of a larger plan, which fill the chip by their number, run their passes
 // one after another

@@ -1,6 +1,5 @@
-// int32 Smith-Waterman wavefront of one warp over one column pass: the exact rescoring of pairs
-// whose int16 scores saturated, and the alignment-cells pass (score plus the first row-major
-// cell reaching it).  Same recurrences as the int16 kernel (Sec. 4's f: affine-gap local
+// int32 Smith-Waterman wavefront of one warp over one column pass: the alignment-cells pass
+// (score plus the first row-major cell reaching it) where scores may reach 2^28.  Same recurrences as the int16 kernel (Sec. 4's f: affine-gap local
 // alignment score), on plain 32-bit integers, so no score range limit.
 //
 // Mapping.  Lane l holds R consecutive columns of the pass (profile segment `plane`, LS words
@@ -31,7 +30,7 @@ __device__ __forceinline__ bool first_max(int32_t b, int32_t r, int32_t c, int32
 }
 
 struct D32Best {
-    int32_t b, r, c;     // score; its first (row, column) in row-major order (CELLS), else -1
+    int32_t b, r, c;     // score; its first (row, column) in row-major order, -1 if 0
 };
 
 // One column pass over rows ra[0..m) (read back to front when `reverse`; m < 2^30).  `bin`:
@@ -39,12 +38,12 @@ struct D32Best {
 // `bout`: where this pass writes its own (nullptr on the last pass).  Before the warp reads the
 // boundary rows [.., need) it calls wait(need) (warp-uniform; false gives up and the pass
 // returns false); lane 31 calls publish(rows) after the first `rows` boundary rows are
-// written.  col0 = the first column of this lane.  CELLS: every row class q (rows = q mod
+// written.  col0 = the first column of this lane.  Every row class q (rows = q mod
 // kD32Rows) keeps its own first maximum with strict > (its rows come in order, a row's columns
 // in order), and the classes, then the lanes, are merged with the row-major tie-break; cells of
 // pad rows or pad columns stay below the maximum over real cells.  Returns the warp's result
 // in `out` on every lane.
-template <int R, int LS, bool CELLS, class Wait, class Publish>
+template <int R, int LS, class Wait, class Publish>
 __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
                                           const uint8_t* __restrict__ ra, int64_t m, bool reverse,
                                           int o, int ge, const int2* bin, int2* bout, int32_t col0,
@@ -62,7 +61,7 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
     int32_t oh[NR], oe[NR], bh[NR], be[NR];               // last column; boundary rows
 #pragma unroll
     for (int q = 0; q < NR; ++q) { oh[q] = -o; oe[q] = -o; bh[q] = -o; be[q] = -o; }
-    int32_t diag0 = -o, best = 0, out_acc = 0, result = 0;
+    int32_t diag0 = -o;
     int32_t lbest[NR], lrow[NR], lcol[NR];
 #pragma unroll
     for (int q = 0; q < NR; ++q) { lbest[q] = 0; lrow[q] = -1; lcol[q] = -1; }
@@ -99,7 +98,6 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
             hL[q] = __shfl_up_sync(kAll, oh[q], 1);
             eL[q] = __shfl_up_sync(kAll, oe[q], 1);
         }
-        int32_t ai = __shfl_up_sync(kAll, out_acc, 1);
         if (bin != nullptr) {
 #pragma unroll
             for (int q = 0; q < NR; ++q) {
@@ -110,7 +108,6 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
 #pragma unroll
             for (int q = 0; q < NR; ++q) { hL[q] = -o; eL[q] = -o; }
         }
-        if (lane == 0) ai = 0;
         int32_t dg[NR], h[NR], e[NR];
         dg[0] = diag0;
 #pragma unroll
@@ -140,11 +137,7 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
                 const int32_t d = __viaddmax_s32(dg[q], sq[q][c & 3], 0);
                 dg[q] = hp[c];
                 const int32_t hh = __vimax3_s32(d, e[q], f);
-                if (CELLS) {
-                    if (hh > lbest[q]) { lbest[q] = hh; lrow[q] = row0 + q; lcol[q] = col0 + c; }
-                } else {
-                    best = max(best, hh);
-                }
+                if (hh > lbest[q]) { lbest[q] = hh; lrow[q] = row0 + q; lcol[q] = col0 + c; }
                 h[q] = hh - o;
                 hp[c] = h[q];
                 fp[c] = f;
@@ -152,10 +145,6 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
         }
 #pragma unroll
         for (int q = 0; q < NR; ++q) { oh[q] = h[q]; oe[q] = e[q]; }
-        if (!CELLS) {
-            out_acc = max(ai, best);
-            if (lane == 31 && t - 31 == ngrp - 1) result = out_acc;
-        }
         if (bout != nullptr && t >= 31 && lane == 31) {
             const int64_t g = (int64_t)(t - 31) * NR;
 #pragma unroll
@@ -168,21 +157,17 @@ __device__ __forceinline__ bool dp32_pass(const int32_t* __restrict__ plane,
         }
     }
     if (bout != nullptr && lane == 31) publish((int32_t)m);
-    if (CELLS) {
-        int32_t b = lbest[0], rw = lrow[0], cl = lcol[0];
+    int32_t b = lbest[0], rw = lrow[0], cl = lcol[0];
 #pragma unroll
-        for (int q = 1; q < NR; ++q)
-            if (first_max(lbest[q], lrow[q], lcol[q], b, rw, cl)) { b = lbest[q]; rw = lrow[q]; cl = lcol[q]; }
-        for (int d = 16; d >= 1; d >>= 1) {
-            const int32_t ob = __shfl_xor_sync(kAll, b, d);
-            const int32_t orw = __shfl_xor_sync(kAll, rw, d);
-            const int32_t oc = __shfl_xor_sync(kAll, cl, d);
-            if (first_max(ob, orw, oc, b, rw, cl)) { b = ob; rw = orw; cl = oc; }
-        }
-        out = D32Best{b, b > 0 ? rw : -1, b > 0 ? cl : -1};
-    } else {
-        out = D32Best{__shfl_sync(kAll, result, 31), -1, -1};
+    for (int q = 1; q < NR; ++q)
+        if (first_max(lbest[q], lrow[q], lcol[q], b, rw, cl)) { b = lbest[q]; rw = lrow[q]; cl = lcol[q]; }
+    for (int d = 16; d >= 1; d >>= 1) {
+        const int32_t ob = __shfl_xor_sync(kAll, b, d);
+        const int32_t orw = __shfl_xor_sync(kAll, rw, d);
+        const int32_t oc = __shfl_xor_sync(kAll, cl, d);
+        if (first_max(ob, orw, oc, b, rw, cl)) { b = ob; rw = orw; cl = oc; }
     }
+    out = D32Best{b, b > 0 ? rw : -1, b > 0 ? cl : -1};
     return true;
 }
 

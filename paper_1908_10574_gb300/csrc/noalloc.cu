@@ -92,7 +92,7 @@ __device__ int32_t na_optimum(const uint8_t* a, int64_t m, const uint8_t* b, int
         wave_profile(prof, a, m, rev, i0, kWaveMaxR, mat, 20, 1, 20);
         __syncwarp();
         int32_t sc, x, y;
-        wave_strip<kWaveMaxR, true>(s, no_wait, no_publish, sc, x, y);
+        wave_strip<kWaveMaxR, kTrackYRows>(s, no_wait, no_publish, sc, x, y);
         if (first_max(sc, y, x, best, row, col)) { best = sc; row = y; col = x; }
     }
     *bi = row + 1;

@@ -1,5 +1,4 @@
-// Launchers of the Smith-Waterman kernels (templates in sw16_kernel.cuh); the int16x2
-// query-pair kernel by CTA width and the int32 rescoring kernel.
+// Launchers of the query-pair kernel of one tile, by CTA width and mode.
 #include "sw16_kernel.cuh"
 
 namespace cm {
@@ -26,19 +25,6 @@ int sw16_ctas_per_sm(int R, int W, int mode)
 #undef CM_OCC_CASE
 }
 
-int sw32_ctas_per_sm()
-{
-    const int smem = sw32_smem_bytes(16);
-    if (cudaFuncSetAttribute(sw32_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) != cudaSuccess)
-        return 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sw32_kernel<16>, 32, smem) !=
-        cudaSuccess)
-        return 1;
-    return n;
-}
-
 cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st)
 {
     if (mode != kModePair && mode != kModeSeg16) return cudaErrorInvalidValue;
@@ -53,24 +39,6 @@ cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaS
     default: return cudaErrorInvalidValue;
     }
 #undef CM_LAUNCH_CASE
-}
-
-int sw32_smem_bytes(int R)
-{
-    const int LS = lane_stride(R);
-    return kProfRows * 32 * LS * 4 + 32 * R;
-}
-
-cudaError_t launch_sw32(int R, int grid, const SwArgs& a, const PairRef* pr, int32_t npairs,
-                        int32_t* counter, cudaStream_t st)
-{
-    if (R != 16) return cudaErrorInvalidValue;
-    const int smem = sw32_smem_bytes(16);
-    cudaError_t e = cudaFuncSetAttribute(sw32_kernel<16>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    sw32_kernel<16><<<grid, 32, smem, st>>>(a, pr, npairs, counter);
-    return cudaGetLastError();
 }
 
 }  // namespace cm

@@ -26,7 +26,6 @@
 #include <algorithm>
 
 #include "cm_internal.h"
-#include "dp32.cuh"
 
 namespace cm {
 
@@ -345,70 +344,6 @@ sw16_kernel(const __grid_constant__ SwArgs a)
                                   ns_lo, ns_hi, T.hi_valid != 0);
             __syncthreads();
         }
-    }
-}
-
-// ---- int32 rescoring of pairs flagged by the int16 pass: one warp per pair -----------------
-// Rows stream the subject x, columns hold the query q in passes of 32 R columns; the passes of
-// a pair run one after another on the warp, the boundary column kept in the warp's own slot
-// of `bnd` (read ahead of where the same pass writes it).
-template <int R>
-__global__ void __launch_bounds__(32) sw32_kernel(const __grid_constant__ SwArgs a,
-                                                 const PairRef* __restrict__ pr,
-                                                 int32_t npairs, int32_t* counter)
-{
-    using G = Geo<R>;
-    extern __shared__ __align__(16) uint8_t smem[];
-    int32_t* prof = reinterpret_cast<int32_t*>(smem);
-    uint8_t* qres = smem + (size_t)G::PROF_WORDS * 4;
-    __shared__ int16_t s_mat[kAlpha * kAlpha];
-    const int lane = threadIdx.x;
-    for (int i = lane; i < kAlpha * kAlpha; i += 32) s_mat[i] = a.mat[i];
-    __syncwarp();
-    const int o = a.gap_open, ge = a.gap_extend;
-    int2* bnd = reinterpret_cast<int2*>(a.bnd + (int64_t)blockIdx.x * a.bnd_stride);
-    auto no_wait = [](int32_t) { return true; };
-    auto no_publish = [](int32_t) {};
-
-    for (;;) {
-        int p = 0;
-        if (lane == 0) p = atomicAdd(counter, 1);
-        p = __shfl_sync(kFull, p, 0);
-        if (p >= npairs) break;
-        const PairRef P = pr[p];
-        const int64_t qoff = a.off[P.q], m = a.off[P.q + 1] - qoff;
-        const int64_t xoff = a.off[P.x];
-        int64_t n = a.off[P.x + 1] - xoff;
-        const int npass = (m <= G::COLS) ? 1 : (int)((m + G::COLS - 1) / G::COLS);
-        if ((npass > 1 && n > a.bnd_stride) || n >= ((int64_t)1 << 30)) {
-            if (lane == 0) atomicExch(a.err, 1);
-            n = 0;
-        }
-        int32_t result = 0;
-        for (int pass = 0; pass < npass && n > 0; ++pass) {
-            const int64_t c0 = (int64_t)pass * G::COLS;
-            __syncwarp();
-            for (int c = lane; c < G::COLS; c += 32)
-                qres[c] = (c0 + c < m) ? a.db[qoff + c0 + c] : kPadCode;
-            __syncwarp();
-            for (int i = lane; i < kProfRows * G::COLS; i += 32) {
-                const int x = i / G::COLS, c = i - x * G::COLS;
-                const int ln = c / R, k = c - ln * R;
-                const int q = qres[c];
-                int s = kSpad;                    // +o: the DP keeps H - o as its diagonal input
-                if (x != kPadCode && q != kPadCode)
-                    s = (P.swap ? s_mat[x * kAlpha + q] : s_mat[q * kAlpha + x]) + o;
-                prof[x * G::ROWW + ln * G::LS + k] = s;
-            }
-            __syncwarp();
-            D32Best r;
-            dp32_pass<R, G::LS, false>(prof + lane * G::LS, a.db + xoff, n, false, o, ge,
-                                       pass > 0 ? bnd : nullptr,
-                                       pass + 1 < npass ? bnd : nullptr,
-                                       (int32_t)c0 + lane * R, no_wait, no_publish, r);
-            result = max(result, r.b);
-        }
-        if (lane == 0) a.out[P.slot] = result;
     }
 }
 

@@ -1,6 +1,6 @@
-// int32 Smith-Waterman wavefront of one warp over one strip, with the first cell that reaches
-// the optimum: the alignment-cells pass.  Same recurrences as the int16 kernel; every score fits
-// (the position key leaves 28 bits, see below).
+// int32 Smith-Waterman wavefront of one warp over one strip: the rescoring of pairs beyond the
+// int16 range, and with the first cell that reaches the optimum the alignment-cells pass.  Same
+// recurrences as the int16 kernel.
 //
 // Mapping.  The matrix is x (streamed) against y (held): lane l holds R consecutive y positions
 // of a strip of 32 R, and at step t works on the 4 x positions of group t - l (x position k of a
@@ -10,15 +10,15 @@
 // Per cell, with the profile holding plain scores as bytes (four per word, pads -128):
 //   E = max(E - e, (H - o)_left),  F = max(F - e, (H - o)_up),
 //   D = H_diag + S (one dp4a: byte select, sign extension and add),  H = max(D, E, F, 0)
-// that is 3 DPX operations and a dot product, then the key 8 H + 7 - (y position in the lane)
-// and half a 3-input maximum over the lane's keys of each x position.  So an x position costs
-// one comparison per lane, not each cell: the largest key says the score and the first y
-// position that has it.
-//   YROWS = false: x are the rows, y the columns of the pair.  A new best needs a larger score;
+// that is 3 DPX operations and a dot product, and half a 3-input maximum of H (kTrackNone) or of
+// the key 8 H + 7 - (y position in the lane) over each x position.  So the position costs one
+// comparison per x position and lane, not per cell: the largest key says the score and the first
+// y position that has it.
+//   kTrackXRows: x are the rows, y the columns of the pair.  A new best needs a larger score;
 //     x positions come in order, so the first row stays.
-//   YROWS = true: y are the rows, x the columns.  A larger key is a larger score or the same
-//     one in an earlier row; an equal key is the same row, whose first column stays.
-// Key range: 8 H + 7 < 2^31, so scores below 2^28 (kWaveScoreLimit).
+//   kTrackYRows: y are the rows, x the columns.  A larger key is a larger score or the same one
+//     in an earlier row; an equal key is the same row, whose first column stays.
+// Key range: 8 H + 7 < 2^31, so tracked scores stay below 2^28 (kWaveScoreLimit).
 #pragma once
 #include <cstdint>
 
@@ -26,6 +26,8 @@
 
 namespace cm {
 namespace {
+
+enum WaveTrack : int { kTrackNone = 0, kTrackXRows = 1, kTrackYRows = 2 };
 
 constexpr int kWaveRows = 4;                      // x positions per step
 constexpr int kWaveProf = kProfRows * 32;         // uint2 entries of a strip's profile
@@ -68,8 +70,9 @@ struct WaveStrip {
 
 // One strip.  wait(groups) returns once the first `groups` groups of bin are written (false gives
 // up: the strip returns false on every lane); lane 31 calls publish(groups) after that many of
-// bout are.  The result, on every lane: score, x and y position of its first cell (-1 if 0).
-template <int R, bool YROWS, class Wait, class Publish>
+// bout are.  The result, on every lane: score, x and y position of its first cell (-1 if 0, or
+// untracked).
+template <int R, int TRACK, class Wait, class Publish>
 __device__ __forceinline__ bool wave_strip(const WaveStrip& s, Wait&& wait, Publish&& publish,
                                            int32_t& score, int32_t& xpos, int32_t& ypos)
 {
@@ -89,7 +92,7 @@ __device__ __forceinline__ bool wave_strip(const WaveStrip& s, Wait&& wait, Publ
     int32_t oh[NR], oe[NR], bh[NR], be[NR];
 #pragma unroll
     for (int q = 0; q < NR; ++q) { oh[q] = -o; oe[q] = -o; bh[q] = -o; be[q] = -o; }
-    int32_t diag0 = -o, lkey = 7, lx = -1;
+    int32_t diag0 = -o, lkey = TRACK != kTrackNone ? 7 : 0, lx = -1;
     constexpr uint32_t kPads = (uint32_t)kPadCode * 0x01010101u;
     uint32_t cur = kPads, prev = kPads;
 
@@ -157,7 +160,7 @@ __device__ __forceinline__ bool wave_strip(const WaveStrip& s, Wait&& wait, Publ
                 const int32_t d = __dp4a((int)(c < 4 ? w[q].x : w[q].y), 1 << (8 * (c & 3)), dg[q]);
                 dg[q] = hp[c] + o;
                 const int32_t hh = __vimax3_s32_relu(d, e[q], f);
-                const int32_t key = hh * 8 + (7 - c);
+                const int32_t key = TRACK != kTrackNone ? hh * 8 + (7 - c) : hh;
                 if (c & 1) best[q] = __vimax3_s32(best[q], pend[q], key);
                 else if (c == R - 1) best[q] = max(best[q], key);
                 else pend[q] = key;
@@ -170,9 +173,13 @@ __device__ __forceinline__ bool wave_strip(const WaveStrip& s, Wait&& wait, Publ
         for (int q = 0; q < NR; ++q) {
             oh[q] = h[q];
             oe[q] = e[q];
-            const bool up = best[q] > (YROWS ? lkey : (lkey | 7));
-            lkey = up ? best[q] : lkey;
-            lx = up ? (t - lane) * NR + q : lx;
+            if (TRACK == kTrackNone) {
+                lkey = max(lkey, best[q]);
+            } else {
+                const bool up = best[q] > (TRACK == kTrackYRows ? lkey : (lkey | 7));
+                lkey = up ? best[q] : lkey;
+                lx = up ? (t - lane) * NR + q : lx;
+            }
         }
         if (bout != nullptr && t >= 31) {                 // (whole groups: bout has room for them)
             if (lane == 31) {
@@ -187,13 +194,18 @@ __device__ __forceinline__ bool wave_strip(const WaveStrip& s, Wait&& wait, Publ
             }
         }
     }
+    if (TRACK == kTrackNone) {
+        score = __reduce_max_sync(kAll, lkey);
+        xpos = ypos = -1;
+        return true;
+    }
     // the lanes' first cells: larger score, then smaller row, then smaller column
     int32_t b = lkey >> 3, px = lx, py = s.y0 + lane * R + 7 - (lkey & 7);
     for (int d = 16; d >= 1; d >>= 1) {
         const int32_t ob = __shfl_xor_sync(kAll, b, d);
         const int32_t ox = __shfl_xor_sync(kAll, px, d);
         const int32_t oy = __shfl_xor_sync(kAll, py, d);
-        if (YROWS ? first_max(ob, oy, ox, b, py, px) : first_max(ob, ox, oy, b, px, py)) {
+        if (TRACK == kTrackYRows ? first_max(ob, oy, ox, b, py, px) : first_max(ob, ox, oy, b, px, py)) {
             b = ob;
             px = ox;
             py = oy;

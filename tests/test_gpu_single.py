@@ -1,7 +1,7 @@
 """The one-warp kernel of lone queries (sw_score_batch's pair lists) at the sizes where it can go
 wrong: tile and pass edges, queries whose column passes run as a pipeline of warps, streams with
-no subject, one subject only, empty sequences, an asymmetric 24-letter matrix.  Scores are
-integers and must equal the oracle's."""
+no subject, one subject only, empty sequences, an asymmetric 24-letter matrix; and the int32
+rescoring of the same pairs.  Scores are integers and must equal the oracle's."""
 import numpy as np
 import pytest
 
@@ -38,5 +38,8 @@ def test_pair_lists_match_oracle(ctx, queries, subjects, alphabet):
     pairs = np.array([(q, nq + s) for q in range(nq) for s in range(len(subjects))] +
                      [(nq + s, q) for s in range(len(subjects)) for q in range(nq)], np.int32)
     S = synth.BLOSUM62 if alphabet == 20 else rng.integers(-9, 10, size=(24, 24)).astype(np.int8)
-    got = ctx.sw_score_batch(ss.seqs, ss.offsets, pairs, S, 11, 1)
-    assert np.array_equal(got, oracle.sw_batch(ss.seqs, ss.offsets, pairs, S, 11, 1))
+    want = oracle.sw_batch(ss.seqs, ss.offsets, pairs, S, 11, 1)
+    assert np.array_equal(ctx.sw_score_batch(ss.seqs, ss.offsets, pairs, S, 11, 1), want)
+    # the same pairs through the int32 strips
+    assert np.array_equal(ctx.sw_score_batch(ss.seqs, ss.offsets, pairs, S, 11, 1,
+                                             flags=cm.CM_FORCE_INT32), want)
