@@ -503,14 +503,15 @@ int conv_tc(cm_ctx* c, Ranker* K, const bf16* X, int64_t R, const bf16* Wk, cons
     using C = tc::ConvCfg<CIN, NOUT>;
     const int64_t tiles = blocks_for(R, tc::kTcRows);
     if (tiles == 0) return CM_OK;
-    CUtensorMap ta, tb;
+    CUtensorMap ta, tb, to{};
     CUDA_TRY(tc::make_tmap_bf16(&ta, X, CIN, (uint64_t)R, C::BK, C::AROWS));
     CUDA_TRY(tc::make_tmap_bf16(&tb, Wk, kTaps * CIN, NOUT, C::BK, NOUT));
+    if (ep.out) CUDA_TRY(tc::make_tmap_bf16(&to, ep.out, NOUT, (uint64_t)R, 64, 32));
     auto kern = tc::conv_tc_kernel<CIN, NOUT, EPI>;
     CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     // persistent: one CTA per SM over the 128-row tiles
     const int grid = (int)std::min<int64_t>(tiles, std::max(1, c->num_sms));
-    kern<<<grid, tc::kConvThreads, C::SMEM, c->stream>>>(ta, tb, R, ep, K->tc_err);
+    kern<<<grid, tc::kConvThreads, C::SMEM, c->stream>>>(ta, tb, to, R, ep, K->tc_err);
     CUDA_TRY(cudaGetLastError());
     c->stats.launches += 1;
     return CM_OK;

@@ -99,6 +99,25 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* m, int
         : "memory");
 }
 
+// store the box at `src` (shared memory, in the map's swizzle) to (x, row y): the rows past the
+// matrix's end are not written.  One bulk group per store.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* src, int32_t x, int32_t y)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];\n"
+                 " cp.async.bulk.commit_group;\n"
+                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_addr(src)) : "memory");
+}
+
+// writes of this thread to shared memory, before a TMA store reads them
+__device__ __forceinline__ void fence_async_proxy()
+{
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+
+// this thread's stores have read their boxes / are complete
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+
 __device__ __forceinline__ uint64_t smem_desc(const void* p, uint32_t lbo, uint32_t sbo,
                                               uint32_t swizzle_mode)
 {
@@ -125,6 +144,27 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                  ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+
+// The same with the descriptors as words: an operand's place moves in the low word only, so a
+// step costs one 32-bit add.
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                         uint32_t bhi, uint32_t idesc, bool accumulate)
+{
+    asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n"
+                 " mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n"
+                 ::"r"(tmem_d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc),
+                   "r"((uint32_t)accumulate) : "memory");
+}
+
+// one thread of a converged warp, always the same.  Code that a whole warp runs around it keeps
+// its values in uniform registers, which the MMA's operands have to be in.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+    return e != 0;
 }
 
 // arrive on `bar` once every tcgen05 operation this thread issued before has completed
