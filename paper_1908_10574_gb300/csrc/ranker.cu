@@ -78,17 +78,6 @@ __global__ void reduce_parts_kernel(const float* __restrict__ part, int64_t nchu
     grad[i] += s;
 }
 
-__global__ void embed_fwd_kernel(const uint8_t* __restrict__ codes, int64_t R,
-                                 const bf16* __restrict__ E, bf16* __restrict__ X0)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= R * kEmb) return;
-    const int64_t r = i / kEmb;
-    const int c = (int)(i % kEmb);
-    const uint8_t code = codes[r];
-    X0[i] = (code < 20) ? E[code * kEmb + c] : __float2bfloat16(0.f);
-}
-
 // pooled vectors from their 64-bit fixed-point sums (units of 2^-32)
 __global__ void fixed_to_float_kernel(const unsigned long long* __restrict__ in, int64_t n,
                                       float* __restrict__ out)
@@ -197,18 +186,123 @@ __global__ void head_kernel(const float* __restrict__ v, const int32_t* __restri
     }
 }
 
-__global__ void gather_rows_kernel(const uint8_t* __restrict__ db, const int64_t* __restrict__ off,
-                                   const int32_t* __restrict__ sid, const int64_t* __restrict__ srow,
-                                   const int32_t* __restrict__ slen, int32_t nseq,
-                                   uint8_t* __restrict__ codes, int32_t* __restrict__ rowseq)
+// Rows of a batch: residue codes (0xff in gap rows), the sequence of each row (-1) and the
+// embedded rows X0 (zero in gap rows and for codes past the 20 embedded ones).  kRowBlocks blocks
+// per sequence write its rows and the gap after them, the first one also the gap before them: every
+// row of the batch, so nothing has to be cleared.  Bound by the stores, 69 bytes a row, 16 per
+// thread: 1.7M rows in 29 us; two memsets, a copy per sequence and a thread per channel of X0
+// took 150.
+constexpr int kRowBlocks = 4;
+
+__global__ void __launch_bounds__(256)
+batch_rows_kernel(const uint8_t* __restrict__ db, const int64_t* __restrict__ off,
+                  const int32_t* __restrict__ sid, const int64_t* __restrict__ srow,
+                  const int32_t* __restrict__ slen, const bf16* __restrict__ E,
+                  uint8_t* __restrict__ codes, int32_t* __restrict__ rowseq, bf16* __restrict__ X0)
 {
+    __shared__ uint4 s_e[21 * 4];                  // 64 bytes a code; code 20: zeros
+    for (int i = threadIdx.x; i < 21 * 4; i += blockDim.x)
+        s_e[i] = i < 80 ? reinterpret_cast<const uint4*>(E)[i] : make_uint4(0, 0, 0, 0);
+    __syncthreads();
     const int s = blockIdx.x;
-    if (s >= nseq) return;
     const uint8_t* src = db + off[sid[s]];
-    const int64_t r0 = srow[s];
-    for (int i = threadIdx.x; i < slen[s]; i += blockDim.x) {
-        codes[r0 + i] = src[i];
-        rowseq[r0 + i] = s;
+    const int len = slen[s], before = s == 0 ? kGap : 0;
+    const int64_t r0 = srow[s] - before;
+    const int rows = before + len + kGap;
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < rows * 4; i += gridDim.y * blockDim.x) {
+        const int r = i >> 2, c = i & 3, p = r - before;
+        const bool real = p >= 0 && p < len;
+        const int code = real ? (int)src[p] : 255;
+        reinterpret_cast<uint4*>(X0)[(r0 + r) * 4 + c] = s_e[min(code, 20) * 4 + c];
+        if (c == 0) codes[r0 + r] = (uint8_t)code;
+        if (c == 1) rowseq[r0 + r] = real ? s : -1;
+    }
+}
+
+// The third layer and the mean pooling of inference, from the second layer's column sums: the
+// layer is linear and so is the mean, so
+//   v[n] = b3[n] + 1/len sum_t sum_c S_t[c] W3[t][c][n],   S_t = sum of Z2[r + t - 4] over the rows
+// of a sequence: the column sum less the 4 - t last rows (t < 4) or the t - 4 first ones.  1,152
+// products per channel and sequence instead of per row: 65 us for 4,000 sequences, where the
+// layer over their 1.7M rows took 361 us and the second one wrote 433 MB for it.
+// One block per kPoolSeqs sequences: the S_t in shared memory (fixed-point differences, exact),
+// each thread two channels of a quarter of K for all of them, FP32.
+constexpr int kPoolSeqs = 8;
+
+__global__ void __launch_bounds__(256)
+pool_linear_kernel(const unsigned long long* __restrict__ sums, const bf16* __restrict__ edge,
+                   const int32_t* __restrict__ slen, int64_t ns, const bf16* __restrict__ W3T,
+                   const float* __restrict__ b3, float* __restrict__ V)
+{
+    __shared__ __align__(16) float S[kTaps * kCh][kPoolSeqs];
+    __shared__ float red[3][kPoolSeqs][kCh];
+    const int64_t s0 = (int64_t)blockIdx.x * kPoolSeqs;
+    for (int i = threadIdx.x; i < kPoolSeqs * kCh; i += blockDim.x) {
+        const int q = i / kCh, c = i % kCh;
+        const int64_t s = s0 + q;
+        const int len = s < ns ? slen[s] : 0;
+        const long long total = len > 0 ? (long long)sums[s * kCh + c] : 0;
+        auto row = [&](int k) {                    // k: 0..3 from the start, 4..7 from the end
+            return to_fixed(__bfloat162float(edge[(s * 8 + k) * kCh + c]));
+        };
+        auto put = [&](int t, long long x) { S[t * kCh + c][q] = (float)x * (float)(1.0 / kPoolScale); };
+        put(4, total);
+        long long lo = total, hi = total;
+        for (int d = 1; d <= 4; ++d) {
+            if (d <= len) {
+                lo -= row(4 + d - 1);              // without the d last rows
+                hi -= row(d - 1);                  // without the d first rows
+            }
+            put(4 - d, lo);
+            put(4 + d, hi);
+        }
+    }
+    __syncthreads();
+    const int n = 2 * (threadIdx.x & 63), slice = threadIdx.x >> 6;
+    float acc[kPoolSeqs][2] = {};
+    constexpr int kPer = kTaps * kCh / 4;          // 288
+    static_assert(kPer % 16 == 0, "whole groups");
+    for (int k0 = slice * kPer; k0 < (slice + 1) * kPer; k0 += 16) {
+        __nv_bfloat162 w2[16];                     // in flight together
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {             // W3T[c][(8 - t) * 128 + n] = W3[t][c][n]
+            const int t = (k0 + u) / kCh, c = (k0 + u) % kCh;
+            w2[u] = *reinterpret_cast<const __nv_bfloat162*>(
+                W3T + (int64_t)c * kTaps * kCh + (kTaps - 1 - t) * kCh + n);
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const float w0 = __bfloat162float(w2[u].x), w1 = __bfloat162float(w2[u].y);
+            float x[kPoolSeqs];
+#pragma unroll
+            for (int h = 0; h < kPoolSeqs; h += 4) {
+                const float4 f = *reinterpret_cast<const float4*>(&S[k0 + u][h]);
+                x[h] = f.x; x[h + 1] = f.y; x[h + 2] = f.z; x[h + 3] = f.w;
+            }
+#pragma unroll
+            for (int q = 0; q < kPoolSeqs; ++q) {
+                acc[q][0] += x[q] * w0;
+                acc[q][1] += x[q] * w1;
+            }
+        }
+    }
+    if (slice > 0)
+#pragma unroll
+        for (int q = 0; q < kPoolSeqs; ++q) {
+            red[slice - 1][q][n] = acc[q][0];
+            red[slice - 1][q][n + 1] = acc[q][1];
+        }
+    __syncthreads();
+    if (slice > 0) return;
+#pragma unroll
+    for (int q = 0; q < kPoolSeqs; ++q) {
+        if (s0 + q >= ns) break;
+        const int len = slen[s0 + q];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float t = acc[q][h] + red[0][q][n + h] + red[1][q][n + h] + red[2][q][n + h];
+            V[(s0 + q) * kCh + n + h] = len > 0 ? t / (float)len + b3[n + h] : 0.f;
+        }
     }
 }
 
@@ -379,7 +473,7 @@ struct Ranker {
 
 enum ActId { A_CODES, A_ROWSEQ, A_X0, A_Z1, A_Z2, A_DZ, A_DY2, A_PART, A_V, A_DV,
              A_SEQ, A_PIDX, A_Y, A_LOGIT, A_EP_SID, A_EP_SROW, A_EP_SLEN, A_EP_PIDX, A_EP_Y,
-             A_V64 };
+             A_V64, A_EDGE };
 
 namespace {
 
@@ -500,7 +594,7 @@ void layout(const Prepared& P, const int32_t* ids, int64_t n, Batch& B)
 template <int CIN, int NOUT, int EPI>
 int conv_tc(cm_ctx* c, Ranker* K, const bf16* X, int64_t R, const bf16* Wk, const ConvEpi& ep)
 {
-    using C = tc::ConvCfg<CIN, NOUT>;
+    using C = tc::ConvCfg<CIN, NOUT, EPI>;
     const int64_t tiles = blocks_for(R, tc::kTcRows);
     if (tiles == 0) return CM_OK;
     CUtensorMap ta, tb, to{};
@@ -511,7 +605,7 @@ int conv_tc(cm_ctx* c, Ranker* K, const bf16* X, int64_t R, const bf16* Wk, cons
     CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     // persistent: one CTA per SM over the 128-row tiles
     const int grid = (int)std::min<int64_t>(tiles, std::max(1, c->num_sms));
-    kern<<<grid, tc::kConvThreads, C::SMEM, c->stream>>>(ta, tb, to, R, ep, K->tc_err);
+    kern<<<grid, tc::conv_threads(CIN), C::SMEM, c->stream>>>(ta, tb, to, R, ep, K->tc_err);
     CUDA_TRY(cudaGetLastError());
     c->stats.launches += 1;
     return CM_OK;
@@ -531,50 +625,61 @@ int check_tc(cm_ctx* c, Ranker* K)
 }
 
 // forward over a batch whose layout (sequence ids, first rows, lengths; R rows) is on the
-// device; leaves X0, Z1, Z2, Z3 and the pooled vectors V on the device
+// device; leaves the pooled vectors V on the device, and with `train` the activations X0, Z1 and
+// Z2 and the row metadata for the backward pass
 int forward_dev(cm_ctx* c, const Prepared& P, Ranker* K, const int32_t* d_sid,
-                const int64_t* d_srow, const int32_t* d_slen, int64_t ns, int64_t R, float** V_out)
+                const int64_t* d_srow, const int32_t* d_slen, int64_t ns, int64_t R, bool train,
+                float** V_out)
 {
     const cudaStream_t st = c->stream;
-    uint8_t* codes; int32_t* rowseq; bf16 *X0, *Z1, *Z2; float* V; unsigned long long* V64;
+    uint8_t* codes; int32_t* rowseq; bf16 *X0, *Z1; float* V; unsigned long long* V64;
     AENSURE(A_CODES, R, codes);
     AENSURE(A_ROWSEQ, R * 4, rowseq);
     AENSURE(A_X0, R * kEmb * 2, X0);
     AENSURE(A_Z1, R * kCh * 2, Z1);
-    AENSURE(A_Z2, R * kCh * 2, Z2);
     AENSURE(A_V, ns * kCh * 4, V);
     AENSURE(A_V64, ns * kCh * 8, V64);
     int r;
-    CUDA_TRY(cudaMemsetAsync(codes, 0xff, R, st));
-    CUDA_TRY(cudaMemsetAsync(rowseq, 0xff, R * 4, st));
     CUDA_TRY(cudaMemsetAsync(V64, 0, ns * kCh * 8, st));
-    gather_rows_kernel<<<(unsigned)ns, 128, 0, st>>>(P.db, P.off, d_sid, d_srow, d_slen, (int32_t)ns,
-                                                     codes, rowseq);
-    embed_fwd_kernel<<<blocks_for(R * kEmb, 256), 256, 0, st>>>(codes, R, K->E, X0);
+    batch_rows_kernel<<<dim3((unsigned)ns, kRowBlocks), 256, 0, st>>>(P.db, P.off, d_sid, d_srow, d_slen, K->E, codes,
+                                                    rowseq, X0);
     CUDA_TRY(cudaGetLastError());
-    c->stats.launches += 2;
+    c->stats.launches += 1;
     ConvEpi ep{};
     ep.rowseq = rowseq;
     ep.bias = K->params + kOffB1;
     ep.out = Z1;
     if ((r = conv_tc<kEmb, kCh, kEpiRelu>(c, K, X0, R, K->W1, ep))) return r;
     ep.bias = K->params + kOffB2;
-    ep.out = Z2;
-    if ((r = conv_tc<kCh, kCh, kEpiRelu>(c, K, Z1, R, K->W2, ep))) return r;
-    // layer 3 is pooled in its epilogue: v = mean over a sequence's rows of conv(Z2) + b3
-    ep.bias = K->params + kOffB3;
-    ep.out = nullptr;
     ep.slen = d_slen;
     ep.acc64 = V64;
-    if ((r = conv_tc<kCh, kCh, kEpiPool>(c, K, Z2, R, K->W3, ep))) return r;
-    fixed_to_float_kernel<<<blocks_for(ns * kCh, 256), 256, 0, st>>>(V64, ns * kCh, V);
+    if (!train) {
+        bf16* edge;
+        AENSURE(A_EDGE, ns * 8 * kCh * 2, edge);
+        ep.out = nullptr;
+        ep.srow = d_srow;
+        ep.edge = edge;
+        if ((r = conv_tc<kCh, kCh, kEpiSum>(c, K, Z1, R, K->W2, ep))) return r;
+        pool_linear_kernel<<<blocks_for(ns, kPoolSeqs), 256, 0, st>>>(V64, edge, d_slen, ns, K->W3T,
+                                                                      K->params + kOffB3, V);
+    } else {
+        bf16* Z2;
+        AENSURE(A_Z2, R * kCh * 2, Z2);
+        ep.out = Z2;
+        if ((r = conv_tc<kCh, kCh, kEpiRelu>(c, K, Z1, R, K->W2, ep))) return r;
+        // layer 3 is pooled in its epilogue: v = mean over a sequence's rows of conv(Z2) + b3
+        ep.bias = K->params + kOffB3;
+        ep.out = nullptr;
+        if ((r = conv_tc<kCh, kCh, kEpiPool>(c, K, Z2, R, K->W3, ep))) return r;
+        fixed_to_float_kernel<<<blocks_for(ns * kCh, 256), 256, 0, st>>>(V64, ns * kCh, V);
+    }
     CUDA_TRY(cudaGetLastError());
     c->stats.launches += 1;
     *V_out = V;
     return CM_OK;
 }
 
-// forward over a batch laid out on the host
+// inference over a batch laid out on the host
 int forward(cm_ctx* c, const Prepared& P, Ranker* K, const Batch& B, float** V_out)
 {
     const int64_t ns = (int64_t)B.sid.size();
@@ -587,7 +692,7 @@ int forward(cm_ctx* c, const Prepared& P, Ranker* K, const Batch& B, float** V_o
     if ((r = copy_in(c, d_sid, B.sid.data(), ns * 4, false))) return r;
     if ((r = copy_in(c, d_srow, B.srow.data(), ns * 8, false))) return r;
     if ((r = copy_in(c, d_slen, B.slen.data(), ns * 4, false))) return r;
-    return forward_dev(c, P, K, d_sid, d_srow, d_slen, ns, B.R, V_out);
+    return forward_dev(c, P, K, d_sid, d_srow, d_slen, ns, B.R, false, V_out);
 }
 
 // weight gradient of a conv layer on the tensor cores: the rows are cut into chunks so that
@@ -694,7 +799,7 @@ int loss_grad_packed(cm_ctx* c, const Prepared& P, Ranker* K, const Packed& B, c
     const int64_t R = B.rows[b];
     const int32_t* d_slen = D.slen + so;
     float* V;
-    int r = forward_dev(c, P, K, D.sid + so, D.srow + so, d_slen, ns, R, &V);
+    int r = forward_dev(c, P, K, D.sid + so, D.srow + so, d_slen, ns, R, true, &V);
     if (r) return r;
     const int32_t* d_pidx = D.pidx + 2 * po;
     const float* d_y = D.y + po;

@@ -31,21 +31,26 @@ namespace cm {
 //              pre-pooling activations are never stored).  The sums are kept in 64-bit fixed
 //              point (units of 2^-32) so that the atomic adds commute: v does not depend on
 //              the order in which CTAs finish, and neither do the ranker's logits.
+//   kEpiSum    colsum[seq] += bf16(relu(acc + bias)) over every real row, in fixed point as Pool;
+//              the rows within 4 of a sequence's ends also go to `edge`, the others nowhere (the
+//              linear third layer needs no more of the second one, see pool_linear_kernel)
 //   kEpiGate   out = bf16(gate > 0 ? acc : 0), and colsum[n] += the column sums of those
 //              values (the bias gradient of the layer below)
 //   kEpiEmbed  dE[code][c] += acc for every real row (the embedding table's gradient; dX0 is
 //              never stored)
-enum Epi : int { kEpiRelu = 0, kEpiPool = 1, kEpiGate = 2, kEpiEmbed = 3 };
+enum Epi : int { kEpiRelu = 0, kEpiPool = 1, kEpiGate = 2, kEpiEmbed = 3, kEpiSum = 4 };
 
 struct ConvEpi {
-    const float* bias;          // Relu, Pool
+    const float* bias;          // Relu, Pool, Sum
     const int32_t* rowseq;      // every mode: sequence index of a row, < 0 for gap rows
     const __nv_bfloat16* gate;  // Gate
     __nv_bfloat16* out;         // Relu, Gate
-    const int32_t* slen;        // Pool: rows of every sequence
+    const int32_t* slen;        // Pool, Sum: rows of every sequence
+    const int64_t* srow;        // Sum: first row of every sequence
+    __nv_bfloat16* edge;        // Sum: ns x 8 x NOUT, rows 0..3 from the start, 0..3 from the end
     const uint8_t* codes;       // Embed: residue code of every row
     float* acc;                 // Gate: column sums; Embed: dE (20 x NOUT)
-    unsigned long long* acc64;  // Pool: v (ns x NOUT) in units of 2^-32
+    unsigned long long* acc64;  // Pool: v, Sum: column sums (ns x NOUT) in units of 2^-32
 };
 
 constexpr double kPoolScale = 4294967296.0;   // 2^32: fixed-point unit of the pooled sums
@@ -96,8 +101,8 @@ __device__ __forceinline__ long long warp_colsum32(long long* v, int lane)
 // One CTA per SM walks the 128-row tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0
 // (one thread) streams the A / B stages of every tile through a ring of STAGES shared-memory
 // stages, across tile boundaries; warp 1 (one thread) issues the MMAs of a tile into one of
-// two TMEM accumulators (tile i uses buffer i & 1) and commits it; warps 2-9 read a finished
-// accumulator back (warp w owns TMEM lanes 32 (w % 4) .., warps w and w + 4 one half of the
+// two TMEM accumulators (tile i uses buffer i & 1) and commits it; warps 2-9 (and 10-17, taking
+// every other tile, in some layers) read a finished accumulator back (warp w owns TMEM lanes 32 (w % 4) .., warps w and w + 4 one half of the
 // columns each) and apply the epilogue while the MMAs of the next tile run, then release the
 // buffer.  What the epilogue needs of its rows (sequence, gate) is loaded before the wait for
 // the MMAs, the bias sits in shared memory, and the results leave through 4 KB of shared memory
@@ -108,37 +113,44 @@ __device__ __forceinline__ long long warp_colsum32(long long* v, int lane)
 // and stops, the others then give up at their next wait, and the teardown waits (bounded) for
 // the copies and MMAs still in flight before the tensor memory is freed.
 constexpr int kConvEpiWarps = 8;    // two per TMEM lane quadrant, each half of the columns
-constexpr int kConvThreads = 64 + 32 * kConvEpiWarps;
+// Groups of epilogue warps: two, taking the tiles in turn, for the 32-channel layer, whose MMAs
+// take a quarter of a 128-channel layer's time and whose epilogue's latency bounds it (1.7M rows:
+// 174 us with one group, 114 with two); one for the others, where more warps slow the issue of
+// the MMAs (the second layer with column sums 382 us with one, 405 with two).
+constexpr int conv_epi_groups(int CIN) { return CIN == 32 ? 2 : 1; }
+constexpr int conv_threads(int CIN) { return 64 + 32 * kConvEpiWarps * conv_epi_groups(CIN); }
 constexpr int kConvStageBudget = 192 * 1024;
 
-template <int CIN, int NOUT>
+template <int CIN, int NOUT, int EPI>
 struct ConvCfg {
     static constexpr int BK = (CIN == 32) ? 32 : 64;       // channels per swizzle row
     static constexpr int KB_PER_TAP = CIN / BK;            // boxes of a tap: one stage holds a tap
-    // AREUSE (128-byte swizzle): a tile's A rows r0 - 4 .. r0 + 131 are loaded once per block
-    // of BK channels, and tap t reads them from row t on (the descriptor start moves by whole
-    // 128-byte rows; the swizzle follows the address, so the shifted view stays valid);
-    // otherwise every stage carries its own 128-row A tile
-    static constexpr bool AREUSE = (BK == 64);
-    static constexpr int AROWS = AREUSE ? kTcRows + 8 : kTcRows;
+    // A tile's A rows r0 - 4 .. r0 + 131 are loaded once per block of BK channels, and tap t reads
+    // them from row t on (the descriptor start moves by whole rows; the swizzle follows the
+    // address, so the shifted view stays valid)
+    static constexpr int AROWS = kTcRows + 8;
     static constexpr int A_BOX_BYTES = AROWS * BK * 2;     // one channel block of a tile
     static constexpr int A_TILE_BYTES = KB_PER_TAP * A_BOX_BYTES;
-    static constexpr int A_SLOTS_BYTES = AREUSE ? 2 * A_TILE_BYTES : 0;   // two tiles in flight
-    static constexpr int A_BYTES = kTcRows * BK * 2;       // A of a stage (no reuse)
+    static constexpr int A_SLOTS = (CIN == 32) ? 4 : 2;    // tiles in flight
+    static constexpr int A_SLOTS_BYTES = A_SLOTS * A_TILE_BYTES;
     static constexpr int B_BOX_BYTES = NOUT * BK * 2;
-    static constexpr int B_BYTES = KB_PER_TAP * B_BOX_BYTES;
-    static constexpr int STAGE_BYTES = (AREUSE ? 0 : A_BYTES) + B_BYTES;
-    static constexpr int STAGES_FIT = (kConvStageBudget - A_SLOTS_BYTES) / STAGE_BYTES;
-    static constexpr int STAGES = STAGES_FIT < 8 ? STAGES_FIT : 8;
+    static constexpr int STAGE_BYTES = KB_PER_TAP * B_BOX_BYTES;     // a tap's weights
+    // RESIDENT: all nine taps' weights fit beside the tiles and are loaded once per CTA;
+    // otherwise they stream through a ring of stages, once per tile
+    static constexpr bool RESIDENT = 9 * STAGE_BYTES <= 80 * 1024;
+    static constexpr int STAGES = RESIDENT ? 9 : (kConvStageBudget - A_SLOTS_BYTES) / STAGE_BYTES;
     static constexpr uint32_t SWZ = (BK == 64) ? kSwizzle128 : kSwizzle64;
     static constexpr uint32_t SBO = 8 * BK * 2;
     static constexpr uint32_t TMEM_COLS = 2 * NOUT < 32 ? 32 : 2 * NOUT;   // two accumulators
     // the embedding-gradient epilogue's scratch: per epilogue warp a 32 x 33 transpose tile
     // and private bins of 20 codes x NOUT channels
     static constexpr int EMB_FLOATS = 4 * (32 * 33 + 20 * NOUT);
-    static constexpr int OUT_BYTES = kConvEpiWarps * 32 * 128;       // 32 rows x 64 channels each
+    static constexpr int GROUPS = conv_epi_groups(CIN);
+    static constexpr int OUT_BYTES =                       // boxes of 32 rows x 64 channels
+        EPI == kEpiRelu || EPI == kEpiGate ? GROUPS * kConvEpiWarps * 32 * 128 : 0;
     static constexpr int SMEM = A_SLOTS_BYTES + STAGES * STAGE_BYTES + OUT_BYTES + 1024;
-    static_assert(A_BOX_BYTES % 1024 == 0 && STAGE_BYTES % 1024 == 0, "1024-byte aligned tiles");
+    static_assert(A_BOX_BYTES % (8 * BK * 2) == 0 && A_SLOTS_BYTES % 1024 == 0 &&
+                  STAGE_BYTES % 1024 == 0, "tiles start on whole swizzle atoms");
 };
 
 // What the epilogue of a tile needs of this thread's row (TMEM lane 32 q + lane), loaded while
@@ -146,6 +158,7 @@ struct ConvCfg {
 struct EpiRow {
     int32_t seq;             // < 0: a gap row, or past the end
     float inv_len;           // Pool
+    int edge_lo, edge_hi;    // Sum: distance to the sequence's first and last row
     int code;                // Embed
     bool binned;
     uint32_t gate[2];        // Gate: bit c = the gate of column 32 j0 + c is open
@@ -158,6 +171,11 @@ __device__ __forceinline__ EpiRow epi_row(int64_t r, int64_t R, int j0, const Co
     const bool in = r < R;
     e.seq = in ? ep.rowseq[r] : -1;
     if (EPI == kEpiPool && e.seq >= 0) e.inv_len = 1.f / (float)ep.slen[e.seq];
+    if (EPI == kEpiSum && e.seq >= 0) {
+        const int64_t pos = r - ep.srow[e.seq];
+        e.edge_lo = (int)min(pos, (int64_t)4);
+        e.edge_hi = (int)min((int64_t)ep.slen[e.seq] - 1 - pos, (int64_t)4);
+    }
     if (EPI == kEpiEmbed) {
         // rows of letters outside the 20 embedded ones (zero embedding) add nothing
         const int code = e.seq >= 0 ? (int)ep.codes[r] : 20;
@@ -193,10 +211,10 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
                                               uint8_t* out)
 {
     const bool real = e.seq >= 0;
-    // Pool: a warp whose real rows all belong to one sequence reduces its 32 rows first
+    // Pool, Sum: a warp whose real rows all belong to one sequence reduces its 32 rows first
     int32_t lead = -1;
     bool one_seq = false;
-    if (EPI == kEpiPool) {
+    if (EPI == kEpiPool || EPI == kEpiSum) {
         lead = __reduce_max_sync(0xffffffffu, e.seq);
         one_seq = __all_sync(0xffffffffu, e.seq < 0 || e.seq == lead);
     }
@@ -221,7 +239,7 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
             __syncwarp();
             continue;
         }
-        if (EPI == kEpiPool || EPI == kEpiRelu) {
+        if (EPI == kEpiPool || EPI == kEpiRelu || EPI == kEpiSum) {
             const float4* b4 = reinterpret_cast<const float4*>(s_bias + n0);
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
@@ -232,9 +250,31 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
                 v[4 * t + 3] += b.w;
             }
         }
-        if (EPI == kEpiPool) {
+        if (EPI == kEpiSum) {
+            uint32_t w[16];
 #pragma unroll
-            for (int t = 0; t < 32; ++t) v[t] = real ? v[t] * e.inv_len : 0.f;
+            for (int t = 0; t < 16; ++t) {
+                const __nv_bfloat162 pr = __floats2bfloat162_rn(real ? fmaxf(v[2 * t], 0.f) : 0.f,
+                                                                real ? fmaxf(v[2 * t + 1], 0.f) : 0.f);
+                w[t] = *reinterpret_cast<const uint32_t*>(&pr);
+                v[2 * t] = __bfloat162float(pr.x);
+                v[2 * t + 1] = __bfloat162float(pr.y);
+            }
+            if (real && min(e.edge_lo, e.edge_hi) < 4) {
+                __nv_bfloat16* dst = ep.edge + (int64_t)e.seq * 8 * NOUT + n0;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const uint4 x = make_uint4(w[4 * t], w[4 * t + 1], w[4 * t + 2], w[4 * t + 3]);
+                    if (e.edge_lo < 4) reinterpret_cast<uint4*>(dst + e.edge_lo * NOUT)[t] = x;
+                    if (e.edge_hi < 4) reinterpret_cast<uint4*>(dst + (4 + e.edge_hi) * NOUT)[t] = x;
+                }
+            }
+        }
+        if (EPI == kEpiPool || EPI == kEpiSum) {
+            if (EPI == kEpiPool) {
+#pragma unroll
+                for (int t = 0; t < 32; ++t) v[t] = real ? v[t] * e.inv_len : 0.f;
+            }
             if (one_seq) {
                 const float t = warp_colsum32(v, lane);
                 if (lead >= 0)
@@ -279,11 +319,11 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
 }
 
 template <int CIN, int NOUT, int EPI>
-__global__ void __launch_bounds__(kConvThreads, 1)
+__global__ void __launch_bounds__(conv_threads(CIN), 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmOut, int64_t R, const ConvEpi ep, int32_t* err)
 {
-    using C = ConvCfg<CIN, NOUT>;
+    using C = ConvCfg<CIN, NOUT, EPI>;
     constexpr int S = C::STAGES;
     constexpr uint32_t IDESC = idesc_bf16_f32(kTcRows, NOUT, false, false);
     // column chunks of 32 per epilogue warp pair; with one chunk only the first four warps
@@ -292,21 +332,23 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t full[S], empty[S], afull[2], aempty[2], tfull[2], tempty[2], done;
+    constexpr int NA = C::A_SLOTS;
+    __shared__ __align__(8) uint64_t full[S], empty[S], afull[NA], aempty[NA], tfull[2], tempty[2], done;
     __shared__ uint32_t tmem_slot;
     __shared__ int32_t s_issued, s_consumed, s_aissued, s_aconsumed, s_abort;
     __shared__ float s_red[EPI == kEpiGate ? NOUT : 1];
-    __shared__ __align__(16) float s_bias[EPI == kEpiRelu || EPI == kEpiPool ? NOUT : 4];
+    constexpr bool BIAS = EPI == kEpiRelu || EPI == kEpiPool || EPI == kEpiSum;
+    __shared__ __align__(16) float s_bias[BIAS ? NOUT : 4];
     constexpr bool STORES = EPI == kEpiRelu || EPI == kEpiGate;
     __shared__ float s_emb[EPI == kEpiEmbed ? C::EMB_FLOATS : 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = (R + kTcRows - 1) / kTcRows;
     if (EPI == kEpiGate)
-        for (int i = threadIdx.x; i < NOUT; i += kConvThreads) s_red[i] = 0.f;
-    if (EPI == kEpiRelu || EPI == kEpiPool)
-        for (int i = threadIdx.x; i < NOUT; i += kConvThreads) s_bias[i] = ep.bias[i];
+        for (int i = threadIdx.x; i < NOUT; i += conv_threads(CIN)) s_red[i] = 0.f;
+    if (BIAS)
+        for (int i = threadIdx.x; i < NOUT; i += conv_threads(CIN)) s_bias[i] = ep.bias[i];
     if (EPI == kEpiEmbed)
-        for (int i = threadIdx.x; i < C::EMB_FLOATS; i += kConvThreads) s_emb[i] = 0.f;
+        for (int i = threadIdx.x; i < C::EMB_FLOATS; i += conv_threads(CIN)) s_emb[i] = 0.f;
 
     if (threadIdx.x == 0) {
         prefetch_tmap(&tmA);
@@ -316,9 +358,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
             mbar_init(&tempty[b], kEpiActive);
-            mbar_init(&afull[b], 1);
-            mbar_init(&aempty[b], 1);
         }
+        for (int a = 0; a < NA; ++a) { mbar_init(&afull[a], 1); mbar_init(&aempty[a], 1); }
         mbar_init(&done, 1);
         fence_mbar_init();
         s_issued = 0;
@@ -335,34 +376,32 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     fence_after_sync();
     const uint32_t tmem = tmem_slot;
 
-    uint8_t* bring = smem + C::A_SLOTS_BYTES;                // B (or A + B) stages
+    uint8_t* bring = smem + C::A_SLOTS_BYTES;                // weight stages
     if (warp == 0) {
         if (lane == 0) {
             // ring position: stage s, phase ph of its barriers; it stages issued so far
             int it = 0, i = 0, s = 0;
             uint32_t ph = 0;
             bool ok = true;
+            auto load_tap = [&](int tap) {
+                mbar_expect_tx(&full[s], C::STAGE_BYTES);
+                for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
+                    tma_load_2d(bring + s * C::STAGE_BYTES + cb * C::B_BOX_BYTES, &tmB,
+                                tap * CIN + cb * C::BK, 0, &full[s]);
+                ++it;
+                if (++s == S) { s = 0; ph ^= 1; }
+            };
             for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++i) {
-                const int32_t r0 = (int32_t)(tile * kTcRows);
-                if constexpr (C::AREUSE) {
-                    const int a = i & 1;
-                    if (i >= 2 && !mbar_wait(&aempty[a], ((i / 2) - 1) & 1, err)) break;
-                    uint8_t* as = smem + a * C::A_TILE_BYTES;
-                    mbar_expect_tx(&afull[a], C::A_TILE_BYTES);
-                    for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
-                        tma_load_2d(as + cb * C::A_BOX_BYTES, &tmA, cb * C::BK, r0 - 4, &afull[a]);
-                }
-                for (int tap = 0; tap < 9; ++tap, ++it) {
+                const int a = i % NA;
+                if (i >= NA && !mbar_wait(&aempty[a], ((i / NA) - 1) & 1, err)) break;
+                mbar_expect_tx(&afull[a], C::A_TILE_BYTES);
+                for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
+                    tma_load_2d(smem + a * C::A_TILE_BYTES + cb * C::A_BOX_BYTES, &tmA, cb * C::BK,
+                                (int32_t)(tile * kTcRows) - 4, &afull[a]);
+                if (C::RESIDENT && i > 0) continue;
+                for (int tap = 0; tap < 9; ++tap) {
                     if (it >= S && !mbar_wait(&empty[s], ph ^ 1, err)) { ok = false; break; }
-                    uint8_t* st = bring + s * C::STAGE_BYTES;
-                    mbar_expect_tx(&full[s], C::STAGE_BYTES);
-                    if constexpr (!C::AREUSE) {
-                        tma_load_2d(st, &tmA, 0, r0 + tap - 4, &full[s]);
-                        st += C::A_BYTES;
-                    }
-                    for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
-                        tma_load_2d(st + cb * C::B_BOX_BYTES, &tmB, tap * CIN + cb * C::BK, 0, &full[s]);
-                    if (++s == S) { s = 0; ph ^= 1; }
+                    load_tap(tap);
                 }
             }
             s_issued = it;
@@ -383,35 +422,45 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint32_t ph = 0;
         bool ok = true;
         for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++i) {
-            const int b = i & 1;
+            const int b = i & 1, a_slot = i % NA;
             if (i >= 2) ok = mbar_wait(&tempty[b], ((i / 2) - 1) & 1, err);
-            if (C::AREUSE) ok = ok && mbar_wait(&afull[b], (i / 2) & 1, err);
+            ok = ok && mbar_wait(&afull[a_slot], (i / NA) & 1, err);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             fence_after_sync();
             const uint32_t acc = tmem + (uint32_t)(b * NOUT);
-            const uint32_t atile = alo + (uint32_t)(b * C::A_TILE_BYTES >> 4);
-            for (int tap = 0; tap < 9; ++tap, ++it) {
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, err)))) break;
-                fence_after_sync();
-                const uint32_t st = slo + (uint32_t)(s * C::STAGE_BYTES >> 4);
-                const uint32_t a = C::AREUSE ? atile + (uint32_t)(tap * C::BK * 2 >> 4) : st;
-                const uint32_t bb = C::AREUSE ? st : st + (uint32_t)(C::A_BYTES >> 4);
+            const uint32_t atile = alo + (uint32_t)(a_slot * C::A_TILE_BYTES >> 4);
+            auto issue_tap = [&](int tap, int st) {
+                const uint32_t a = atile + (uint32_t)(tap * C::BK * 2 >> 4);
+                const uint32_t w = slo + (uint32_t)(st * C::STAGE_BYTES >> 4);
+#pragma unroll
+                for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
+#pragma unroll
+                    for (int k = 0; k < C::BK / 16; ++k)
+                        mma_bf16(acc, a + (cb * C::A_BOX_BYTES >> 4) + 2 * k, hi,
+                                 w + (cb * C::B_BOX_BYTES >> 4) + 2 * k, hi, IDESC,
+                                 k > 0 || cb > 0 || tap > 0);
+            };
+            if (C::RESIDENT && i > 0) {           // every tap's weights are there
                 if (elect_one()) {
 #pragma unroll
-                    for (int cb = 0; cb < C::KB_PER_TAP; ++cb)
-#pragma unroll
-                        for (int k = 0; k < C::BK / 16; ++k)
-                            mma_bf16(acc, a + (cb * C::A_BOX_BYTES >> 4) + 2 * k, hi,
-                                     bb + (cb * C::B_BOX_BYTES >> 4) + 2 * k, hi, IDESC,
-                                     k > 0 || cb > 0 || tap > 0);
-                    mma_commit(&empty[s]);
+                    for (int tap = 0; tap < 9; ++tap) issue_tap(tap, tap);
                 }
                 __syncwarp();
-                if (++s == S) { s = 0; ph ^= 1; }
+            } else {
+                for (int tap = 0; tap < 9; ++tap, ++it) {
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, err)))) break;
+                    fence_after_sync();
+                    if (elect_one()) {
+                        issue_tap(tap, s);
+                        mma_commit(&empty[s]);
+                    }
+                    __syncwarp();
+                    if (++s == S) { s = 0; ph ^= 1; }
+                }
             }
             if (!ok) break;
             if (elect_one()) {
-                if (C::AREUSE) mma_commit(&aempty[b]);
+                mma_commit(&aempty[a_slot]);
                 mma_commit(&tfull[b]);
             }
             __syncwarp();
@@ -422,16 +471,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             mma_commit(&done);            // arrives once every MMA issued above has completed
         }
         __syncwarp();
-    } else if (warp - 2 < kEpiActive) {
-        const int ew = warp - 2;
+    } else if ((warp - 2) % kConvEpiWarps < kEpiActive) {
+        const int group = (warp - 2) / kConvEpiWarps, ew = (warp - 2) % kConvEpiWarps;
         const int q = warp & 3;           // TMEM lane quadrant of this warp
         const int half = kEpiActive == 8 ? ew / 4 : 0;
         const int j0 = kEpiActive == 8 ? half * (NCH / 2) : 0;
         const int j1 = kEpiActive == 8 ? (half + 1) * (NCH / 2) : NCH;
         float* emb = s_emb + (EPI == kEpiEmbed ? ew * (32 * 33 + 20 * NOUT) : 0);
-        uint8_t* out = bring + S * C::STAGE_BYTES + ew * (32 * 128);
-        int i = 0;
-        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
+        uint8_t* out = bring + S * C::STAGE_BYTES + (warp - 2) * (32 * 128);
+        int i = group;
+        for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < ntiles;
+             tile += (int64_t)C::GROUPS * gridDim.x, i += C::GROUPS) {
             const int b = i & 1;
             const int64_t row0 = tile * kTcRows + q * 32;
             const EpiRow er = epi_row<NOUT, EPI>(row0 + lane, R, j0, ep);
@@ -462,19 +512,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         mbar_wait(&done, 0, err);
         for (int it = s_consumed; it < s_issued; ++it)
             mbar_wait(&full[it % S], (it / S) & 1, err);
-        if (C::AREUSE)
-            for (int i = s_aconsumed; i < s_aissued; ++i)
-                mbar_wait(&afull[i & 1], (i / 2) & 1, err);
+        for (int i = s_aconsumed; i < s_aissued; ++i) mbar_wait(&afull[i % NA], (i / NA) & 1, err);
     }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     if (EPI == kEpiGate && ep.acc)
-        for (int i = threadIdx.x; i < NOUT; i += kConvThreads)
+        for (int i = threadIdx.x; i < NOUT; i += conv_threads(CIN))
             if (s_red[i] != 0.f) atomicAdd(ep.acc + i, s_red[i]);
     if (EPI == kEpiEmbed) {
         const int per = 32 * 33 + 20 * NOUT;
-        for (int i = threadIdx.x; i < 20 * NOUT; i += kConvThreads) {
+        for (int i = threadIdx.x; i < 20 * NOUT; i += conv_threads(CIN)) {
             float t = 0.f;
 #pragma unroll
             for (int w = 0; w < 4; ++w) t += s_emb[w * per + 32 * 33 + i];
