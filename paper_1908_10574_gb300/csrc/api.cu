@@ -332,6 +332,11 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     a.gap_open = P.g1;
     a.gap_extend = P.ge;
     a.beta = P.beta;
+    a.beta2 = (uint32_t)P.beta * 0x10001u;
+    a.open2 = (uint32_t)P.g1 * 0x10001u;
+    a.bmo2 = a.beta2 - a.open2;
+    a.ext2 = (uint32_t)P.ge * 0x10001u;
+    a.nege2 = (uint32_t)(uint16_t)-P.ge * 0x10001u;
     a.sat_thr = (flags & CM_FORCE_INT32) ? -1 : P.sat_thr;   // -1: every pair goes to int32
 
     // Launches.  All single-query tasks run in one launch, each CTA a contiguous range of them

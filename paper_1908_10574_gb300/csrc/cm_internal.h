@@ -119,6 +119,9 @@ struct SwArgs {
     int16_t mat[kAlpha * kAlpha];   // substitution matrix, [first residue][second residue]
     int32_t gap_open;           // first-gap cost (already includes extend for BLAST mode)
     int32_t gap_extend;
+    // the same constants in both halves of a word, as kernel parameters: the query-pair kernels'
+    // inner loop takes them as operands without a register (or its read port)
+    uint32_t beta2, bmo2, open2, ext2, nege2;   // beta, beta - o, o, e, -e
     int32_t beta;               // int16 bias: stored = true + beta
     int32_t sat_thr;            // stored best >= sat_thr -> rerun in int32
     int32_t wait_limit;         // polls of a bounded device wait before it gives up (long pairs)

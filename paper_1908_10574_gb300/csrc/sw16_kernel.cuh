@@ -14,14 +14,29 @@
 // per pair.  The two 16-bit halves of every register carry two different queries that share
 // the subject stream, so each packed DPX instruction advances two cells.
 //
-// Packed-int16 formulation.  Every stored value carries a bias beta >= o+e (stored = true +
-// beta), which keeps each half within [beta-o, 32767].  The DP keeps H - o, the value both gap
-// types open from, and the profile carries S + o, so the diagonal term reads H - o as well:
-// per packed column 3 viaddmax (E, F, diagonal), 1 vimax3 (H) and 1/2 vimax3 (running
-// maximum, every two columns) on the ALU pipe, plus one plain 32-bit subtract for H - o on
-// the IADD path (H >= beta > o in both halves, so it never borrows across them).  If a stored
-// best reaches 32767 - max(S), some cell may have overflowed int16; that pair is marked and
-// rescored on the int32 path, so every score returned is exact.
+// Packed-int16 formulation.  Every stored value carries a bias beta >= max(o + e, -min S) + 1
+// (stored = true + beta), which keeps each half within [beta - o, 32767].  The DP keeps H - o,
+// the value both gap types open from, and the profile carries S + o, so the diagonal term reads
+// H - o as well.  Per packed column (two cells):
+//   E = viaddmax(E, -e, (H - o)_left)           F = vimax3(F - e, (H - o)_up, beta)
+//   D = (H - o)_diag + (S + o)                  H = vimax3(D, E, F), then H - o
+//   and half a vimax3 for the running maximum (every two columns).
+// The floor beta sits in F, whose add is a plain one, instead of in D: an F below it is worth no
+// more than a local alignment's start, which H takes from F then.  So three of the adds (F - e, D,
+// H - o) are plain 32-bit adds of both halves, which issue beside the ALU pipe, and 3.5 operations
+// are left on it (4.5 with the floor in D = viaddmax(..., beta)).  None of the three carries or
+// borrows between the halves: F >= beta > e and H >= beta > o, so the differences stay positive;
+// H + S >= beta + min S >= 1 and <= 32767 + 127 < 65536, so D's low half neither borrows (a
+// negative S + o is spread over the word, addend2) nor carries, also past the point where a half
+// has left int16 and reads as negative: H takes F there.
+// If a stored best reaches 32767 - max(S), some cell may have overflowed int16; that pair is
+// marked and rescored on the int32 path, so every score returned is exact.
+//
+// Bound: dispatch.  On a set of 350 residues (22 columns a lane) the ALU pipe is 71 % busy, the
+// pipe of the plain adds 65 %, and instructions issue in 74 % of the cycles; with D on the ALU pipe
+// it was 85 % busy and 63 % issued.  The constants are kernel parameters, which take no register
+// and no read port: with them in registers the same update was 4 % slower than D on the ALU pipe.
+// One sixteenth of the 20,000-protein triangle: 319 -> 307 ms per call.
 #pragma once
 #include <algorithm>
 
@@ -32,7 +47,6 @@ namespace cm {
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr int kSpad = -1024;   // profile entry of pad rows / pad columns (any value <= 0 works)
 
 // Tile geometry: SEG lanes (32, or 16 for a half-warp segment) of R columns each.
 template <int R, int SEG = 32>
@@ -46,6 +60,13 @@ struct Geo {
 __device__ __forceinline__ uint32_t pack2(int lo, int hi)
 {
     return (uint32_t)(uint16_t)(int16_t)lo | ((uint32_t)(uint16_t)(int16_t)hi << 16);
+}
+
+// profile word of two halves for a plain 32-bit add: lo + 65536 hi, so that a negative low half
+// borrows what its sum with a larger value carries
+__device__ __forceinline__ uint32_t addend2(int lo, int hi)
+{
+    return (uint32_t)lo + ((uint32_t)hi << 16);
 }
 
 __device__ __forceinline__ int64_t tri(int64_t k) { return k * (k - 1) / 2; }
@@ -126,11 +147,8 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
     using G = Geo<R, SEG>;
     constexpr int NR = kRowGroup;
     const int lane = threadIdx.x & (SEG - 1);    // lane within the segment
-    const int o = a.gap_open, ge = a.gap_extend, beta = a.beta;
-    const uint32_t BETA2 = (uint32_t)beta * 0x10001u;
-    const uint32_t BMO2 = (uint32_t)(beta - o) * 0x10001u;   // H - o of an empty prefix; E, F floor
-    const uint32_t O2 = (uint32_t)o * 0x10001u;
-    const uint32_t NEGE = pack2(-ge, -ge);
+    const uint32_t BETA2 = a.beta2, O2 = a.open2, E2 = a.ext2, NEGE = a.nege2;
+    const uint32_t BMO2 = a.bmo2;                 // H - o of an empty prefix; E, F floor
     constexpr uint32_t PADW = kPadCode * 0x01010101u;
     // boundary records of one step: (H - o, E) of the last column of each of its rows, as
     // uint4 pairs of rows
@@ -218,10 +236,7 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
         uint32_t sq[NR][4];
         uint32_t pend = 0;
         bool has_pend = false;
-        // Row q trails row q-1 by one column.  Per packed cell: E = max(E - e, (H - o)_left),
-        // F = max(F - e, (H - o)_up), D = max((H - o)_diag + (S + o), beta), H = max(D, E, F),
-        // then H - o once for the neighbours (plain 32-bit subtract: H >= beta >= o + e, so
-        // neither half borrows).
+        // row q trails row q-1 by one column; the recurrences are at the top of the file
 #pragma unroll
         for (int k = 0; k < R + NR - 1; ++k) {
 #pragma unroll
@@ -230,8 +245,8 @@ __device__ __forceinline__ void warp_dp16(const SwArgs& a, const SwBlock& B,
                 if (c < 0 || c >= R) continue;
                 if ((c & 3) == 0) load_cols<R>(prow[q], c, sq[q]);   // next profile columns
                 e[q] = __viaddmax_s16x2(e[q], NEGE, h[q]);
-                const uint32_t f = __viaddmax_s16x2(fp[c], NEGE, hp[c]);
-                const uint32_t d = __viaddmax_s16x2(dg[q], sq[q][c & 3], BETA2);
+                const uint32_t f = __vimax3_s16x2(fp[c] - E2, hp[c], BETA2);
+                const uint32_t d = dg[q] + sq[q][c & 3];
                 dg[q] = hp[c];
                 const uint32_t hh = __vimax3_s16x2(d, e[q], f);
                 if (has_pend) { best = __vimax3_s16x2(best, pend, hh); has_pend = false; }
@@ -331,12 +346,12 @@ sw16_kernel(const __grid_constant__ SwArgs a)
                 const int x = i / G::COLS, c = i - x * G::COLS;
                 const int ln = c / R, k = c - ln * R;
                 const int ql = qres[c], qh = qres[G::COLS + c];
-                int sl = kSpad, sh = kSpad;
+                int sl = 0, sh = 0;           // pads score -o
                 if (x != kPadCode) {          // +o: the DP keeps H - o as its diagonal input
                     if (ql != kPadCode) sl = (B.swap ? s_mat[x * kAlpha + ql] : s_mat[ql * kAlpha + x]) + a.gap_open;
                     if (qh != kPadCode) sh = (B.swap ? s_mat[x * kAlpha + qh] : s_mat[qh * kAlpha + x]) + a.gap_open;
                 }
-                prof[x * G::ROWW + ln * G::LS + k] = pack2(sl, sh);
+                prof[x * G::ROWW + ln * G::LS + k] = addend2(sl, sh);
             }
             __syncthreads();
             if (nmax > 0)

@@ -56,9 +56,9 @@ __device__ __forceinline__ void pair_task(const SwArgs& a, const SwTask& T, cons
             const int ln = c / R;
             uint32_t* out = prof + ln * G::LS + (c - ln * R);
             for (int x = 0; x < kAlpha; ++x)
-                out[x * G::ROWW] = pack2(ql != kPadCode ? s_mat[ql * qs + x * xs] + a.gap_open : kSpad,
-                                         qh != kPadCode ? s_mat[qh * qs + x * xs] + a.gap_open : kSpad);
-            out[kPadCode * G::ROWW] = pack2(kSpad, kSpad);
+                out[x * G::ROWW] = addend2(ql != kPadCode ? s_mat[ql * qs + x * xs] + a.gap_open : 0,
+                                           qh != kPadCode ? s_mat[qh * qs + x * xs] + a.gap_open : 0);
+            out[kPadCode * G::ROWW] = 0;          // pads score -o
         }
         __syncthreads();
         if (nmax > 0)
