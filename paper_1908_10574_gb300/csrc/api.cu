@@ -429,8 +429,11 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         }
     }
     int pair_smem = 0;
+    int bins = 0;                                 // the tasks come bin by bin
+    for (size_t i = 0; i < plan.tasks.size(); ++i)
+        bins += i == 0 || plan.task_R[i] != plan.task_R[i - 1];
     const bool one_pairs = W == 16 && launch_sw16_pairs && !plan.tasks.empty() &&
-                           (int64_t)plan.tasks.size() <= (int64_t)kMergedTasks * c->num_sms;
+                           (double)plan.tasks.size() <= kMergedTasks * bins * c->num_sms;
     if (one_pairs) {                              // longest first, whatever their tile
         const size_t n = plan.tasks.size();
         std::vector<std::pair<int64_t, size_t>> order(n);

@@ -97,7 +97,9 @@ constexpr int kProgWords = 4;
 // the long queries of a larger plan, which fill the chip by their number, run their passes
 // one after another
 constexpr int64_t kPipedRows = (int64_t)1 << 26;
-constexpr int kMergedTasks = 64;   // query-pair tasks per SM up to which one launch takes all tiles
+// A plan of query pairs takes one launch for all its tiles up to this many tasks per SM and
+// launch bin (sw16_pair.cu gives the reason)
+constexpr double kMergedTasks = 1.5;
 constexpr int kTaskBins = 32 * 4;
 constexpr int kFlagWords = 8 + kTaskBins;
 

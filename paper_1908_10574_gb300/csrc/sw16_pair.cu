@@ -2,13 +2,14 @@
 // of a plan too small to fill the chip tile by tile.  The tile is a field of the task; a CTA of
 // 16 warps fills an SM whatever its tile.
 //
-// For plans of up to kMergedTasks tasks per SM.  With a launch per tile (sw16_kernel), two at a
-// time, the 20 to 48 tiles of such a plan ran one after another on a dozen CTAs each: the
-// all-against-all of 200 proteins took 4.8 ms, ClusterMerge of 3,000 proteins 440 ms; in one
-// launch 1.7 and 91 ms.  In large plans, where every tile fills the chip, the
-// kernels of one tile are 4 to 6 % faster (one sixteenth of the 20,000-protein triangle, 30,000
-// tasks: 315 ms against 327 to 333 ms): their row loops share no register budget and no
-// instruction cache with other tiles'.
+// For plans of up to kMergedTasks tasks per SM and tile.  A launch per tile (sw16_kernel), two at a
+// time, leaves SMs idle at the end of each: with the 20 to 48 tiles of a small plan most of the
+// chip (all-against-all of 200 proteins 4.7 ms against 1.7 in one launch, of 2,000 in two parts 59
+// against 27, ClusterMerge of 3,000 proteins 440 against 91).  Where a tile has enough tasks the
+// kernels of one tile are 3 to 7 % faster, as their row loops share no register budget and no
+// instruction cache with other tiles'.  The line, measured at one launch / a launch per tile, in
+// ms: 4,000 proteins whole (some 45 tiles) 200 / 216, in 2 parts 99.2 / 111, in 4 (fewer lengths
+// each) 51.8 / 49.8; 7,000 in 4 parts 160 / 155; a 32nd of 20,000 (two or three tiles) 171 / 160.
 #include "sw16_kernel.cuh"
 
 namespace cm {
