@@ -785,19 +785,17 @@ int run_cells(cm_ctx* c, const Prepared& P, const int32_t* hp, int64_t n_pairs, 
     if (n_pairs >= ((int64_t)1 << 31)) return fail(c, CM_ERR_ARG, "n_pairs must be < 2^31");
     const cudaStream_t st = c->stream;
     // long jobs first (a launch of their own, its waits bounded by cm_set_wait_limit), then the
-    // rest, each longest first; pad = the pair's index
+    // rest, each longest first (to within a cost bucket); pad = the pair's index
     auto is_long = [](const CellJob& x) { return x.n >= kLongMinCols && x.m >= kLongMinRows; };
     std::vector<CellJob> jobs((size_t)n_pairs);
     {
-        std::vector<std::pair<int64_t, int32_t>> key((size_t)n_pairs);
-        for (int64_t k = 0; k < n_pairs; ++k) {
-            const int64_t m = P.len(hp[2 * k]), n = P.len(hp[2 * k + 1]);
-            key[k] = {-m * n, (int32_t)k};
-        }
-        std::sort(key.begin(), key.end());
+        const std::vector<int64_t> ord = counting_order(n_pairs, kCostBuckets, [&](int64_t k) {
+            return cost_bucket(P.len(hp[2 * k]) * P.len(hp[2 * k + 1]));
+        });
         for (int64_t q = 0; q < n_pairs; ++q) {
-            const int32_t k = key[q].second, x = hp[2 * (int64_t)k], y = hp[2 * (int64_t)k + 1];
-            jobs[q] = CellJob{x, y, (int32_t)P.len(x), (int32_t)P.len(y), 0, k};
+            const int64_t k = ord[q];
+            const int32_t x = hp[2 * k], y = hp[2 * k + 1];
+            jobs[q] = CellJob{x, y, (int32_t)P.len(x), (int32_t)P.len(y), 0, (int32_t)k};
         }
         std::stable_partition(jobs.begin(), jobs.end(), is_long);
     }
@@ -1063,11 +1061,8 @@ int sw_score_batch(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int32
         if (hp[k] < 0 || hp[k] >= n_seqs) return fail(c, CM_ERR_ARG, "pair index out of range");
 
     // group pairs by their first sequence: one CROSS block {a} x {b...} per distinct a
-    std::vector<int64_t> ord((size_t)n_pairs);
-    std::iota(ord.begin(), ord.end(), 0);
-    std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) {
-        return hp[2 * x] < hp[2 * y];
-    });
+    const std::vector<int64_t> ord =
+        counting_order(n_pairs, n_seqs, [&](int64_t k) { return (int64_t)hp[2 * k]; });
     Plan plan;
     std::vector<int32_t> a_ids, b_ids;
     std::vector<int64_t> omap((size_t)n_pairs);
