@@ -61,7 +61,7 @@ T_SIG = 100
 M_T, M_U = 138, 15
 GAP_OPEN, GAP_EXT = 11, 1
 PARTS_PER_GPU = 16
-OPS_PER_PACKED_CELL = 4.5    # DPX/ALU-pipe operations of the kernel's cell update, 2 cells each
+OPS_PER_PACKED_CELL = 3.5    # DPX/ALU-pipe operations of the kernel's cell update, 2 cells each
 OPS_PER_PACKED_CELL_PLAIN = 7.0   # the plain per-cell count (E 2, F 2, H 2, running max 1)
 
 
