@@ -32,11 +32,12 @@
 // If a stored best reaches 32767 - max(S), some cell may have overflowed int16; that pair is
 // marked and rescored on the int32 path, so every score returned is exact.
 //
-// Bound: dispatch.  On a set of 350 residues (22 columns a lane) the ALU pipe is 71 % busy, the
-// pipe of the plain adds 65 %, and instructions issue in 74 % of the cycles; with D on the ALU pipe
-// it was 85 % busy and 63 % issued.  The constants are kernel parameters, which take no register
-// and no read port: with them in registers the same update was 4 % slower than D on the ALU pipe.
-// One sixteenth of the 20,000-protein triangle: 319 -> 307 ms per call.
+// Bound: the ALU pipe (75 % busy) and the pipe of the plain adds (69 %) together, with 79 % of the
+// issue slots used: 1,200 sequences of 350 residues, 11.7 ms.  With D on the ALU pipe that pipe
+// was 85 % busy, 63 % of the slots were used, and the set took 12.8 ms.  The constants are kernel
+// parameters, which take no register and no read port: with them in registers this update was 4 %
+// slower than D on the ALU pipe.  One sixteenth of the 20,000-protein triangle: 319 -> 307 ms per
+// call.
 #pragma once
 #include <algorithm>
 
