@@ -169,11 +169,12 @@ __device__ __forceinline__ bool align_fill(const AlnJob& J, const uint8_t* __res
 #pragma unroll
                 for (int k = 0; k < kAlnRows; ++k)
                     if (row0 + k < p) __stcg(bnd + row0 + k, make_int2(oh[k], oe[k]));
-                if (j == 31) publish_groups(progress, t - 30);
+                const int32_t done = groups_after_step(t, groups);
+                if (done > 0) publish_groups(progress, done);
             }
         }
     }
-    // all of this pass's directions are written before the last groups are published
+    // all lanes' directions of this pass are written before its last group is published
     __threadfence();
     __syncwarp();
     if (lane == 31 && pass + 1 < npass) publish_groups(progress, groups);

@@ -161,6 +161,13 @@ inline __host__ __device__ int32_t wave_R(int64_t n)
     return per <= 0 ? 1 : (int32_t)((per + 31) / 32);
 }
 inline __host__ __device__ int32_t cell_strips(int64_t m, int64_t n) { return m <= 0 ? 1 : wave_strips(n); }
+// Row groups of a boundary column that a pass of one warp publishes after step t of its wavefront
+// (lane 31 is 31 groups behind): 1, 33, 65, ..., and 0 for none.  Never the last group: the pass
+// publishes that one itself, behind a fence, once everything else it hands on is written.
+inline __host__ __device__ int32_t groups_after_step(int32_t t, int32_t groups)
+{
+    return (t & 31) == 31 && t - 30 < groups ? t - 30 : 0;
+}
 struct CellUnit {
     int32_t job, strip;
     int32_t limit;                     // polls of its wait for the strip before
