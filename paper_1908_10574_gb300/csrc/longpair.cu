@@ -96,6 +96,7 @@ huge_cells_kernel(const __grid_constant__ SwArgs a, const CellJob* __restrict__ 
                     }
                     __threadfence_block();
                 }
+                __syncwarp();                     // orders the other lanes' reads too
                 return __shfl_sync(0xffffffffu, ok, 0) != 0;
             };
             auto publish = [&](int32_t rows) {

@@ -12,7 +12,9 @@ namespace cm {
 namespace {
 
 // waits (lane 0 polls) until `need` row groups are written; false on every lane once `limit`
-// polls have passed, or when another wait has given up and set `err`
+// polls have passed, or when another wait has given up and set `err`.  Lane 0's acquire orders
+// only what lane 0 does next; the barrier after it passes that order on to the lanes that read
+// the rows (a shuffle does not).
 __device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, const int32_t* err,
                                             int32_t limit = kPollLimit)
 {
@@ -30,6 +32,7 @@ __device__ __forceinline__ bool wait_groups(const int32_t* done, int32_t need, c
             __nanosleep(100);
         }
     }
+    __syncwarp();
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
