@@ -80,9 +80,10 @@ struct SwTask {
 };
 
 // One work unit of the single-query launch: a task's passes [pass, pass_end).  A unit with all
-// passes runs them one after another over its warp's boundary slot.  A unit of one pass of
-// several (a pipelined task: its passes are consecutive units) reads and then overwrites, row
-// by row, the boundary column that the unit before it writes at piped + bnd_row.
+// passes runs them one after another over its warp's boundary slot, in pieces of its subjects
+// that fit the slot (piece_end).  A unit of one pass of several (a pipelined task: its passes are
+// consecutive units) reads and then overwrites, row by row, the boundary column that the unit
+// before it writes at piped + bnd_row.
 struct SwUnit {
     int32_t block, k, s0, s1;
     int32_t npass, pass, pass_end;
@@ -90,6 +91,20 @@ struct SwUnit {
     int32_t rows;       // pipelined: rows of the boundary column
     int64_t bnd_row;    // pipelined: its first row in SwArgs::piped, else -1
 };
+
+// End of the piece of subjects [s0, s1) that a unit of several passes runs at once over a boundary
+// slot of `slot` rows: as many whole subjects as have that many rows together (so no split of them
+// over streams is longer), one at least.  A task's rows are only about its target where its list
+// was cut by count (device-built lists), so a run of long subjects may be several pieces.
+inline __host__ __device__ int32_t piece_end(const int64_t* srow, int32_t s0, int32_t s1, int64_t slot)
+{
+    int32_t lo = s0 + 1, hi = s1;                  // the last end in [lo, hi] that fits
+    while (lo < hi) {
+        const int32_t mid = lo + (hi - lo + 1) / 2;
+        if (srow[mid] - srow[s0] <= slot) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
 
 struct CellUnit;
 

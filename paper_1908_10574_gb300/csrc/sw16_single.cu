@@ -284,57 +284,60 @@ sw16_single_kernel(const __grid_constant__ SwArgs a)
         const int64_t* srow = a.srows + B->srow;
         const bool two16 = T.mode == kModeTwo16;
         const int ns = two16 ? 4 : 2;
-        // the streams' boundaries, and this lane's two streams
-        const int64_t R0 = srow[T.s0], R1 = srow[T.s1];
+        const int seg = two16 ? 16 : 32;
         const int i_lo = two16 ? 2 * (lane >> 4) : 0;
-        int32_t at[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-            at[i] = nearest_boundary(srow, T.s0, T.s1, R0 + (R1 - R0) * (i_lo + i) / ns);
+        const bool piped = T.bnd_row >= 0;
         SingleArgs t;
         t.B = B;
-        t.st_lo = reinterpret_cast<const uint32_t*>(a.streams + B->stream + srow[at[0]]);
-        t.st_hi = reinterpret_cast<const uint32_t*>(a.streams + B->stream + srow[at[1]]);
-        t.g_lo = (int32_t)((srow[at[1]] - srow[at[0]]) / kRows);
-        t.g_hi = (int32_t)((srow[at[2]] - srow[at[1]]) / kRows);
-        t.g_max = __reduce_max_sync(kFull, max(t.g_lo, t.g_hi));
-        t.s_lo = at[0];
-        t.s_hi = at[1];
         t.k = T.k;
         t.ns = (B->kind == kTri) ? T.k : B->nb;
         t.npass = T.npass;
-        const bool piped = T.bnd_row >= 0;
         t.bnd = piped ? reinterpret_cast<uint4*>(a.piped + T.bnd_row) : bnd;
         t.err = a.err;
-        if (T.npass > 1 && (int64_t)t.g_max * kRows > (piped ? T.rows : a.bnd_stride)) {
-            if (lane == 0) atomicExch(a.err, 1);  // boundary buffer too small: refuse
-            continue;
-        }
-        const int seg = two16 ? 16 : 32;
-        for (int pass = T.pass; pass < T.pass_end; ++pass) {
-            t.pass = pass;
-            t.done_in = piped && pass > 0 ? a.progress + ti - 1 : nullptr;
-            t.done_out = piped && pass + 1 < T.npass ? a.progress + ti : nullptr;
-            __syncwarp();
-            build_profile(a.db + qoff, m, (int64_t)pass * seg * T.R, T.R, seg, s_mat,
-                          B->swap ? 1 : MS, B->swap ? MS : 1, smem + warp * kSingleSmem);
-            if (two16) {
-                switch (T.R) {
+        for (int32_t s0 = T.s0, s1; s0 < T.s1; s0 = s1) {
+            s1 = piped || T.npass == 1 ? T.s1 : piece_end(srow, s0, T.s1, a.bnd_stride);
+            // the streams' boundaries, and this lane's two streams
+            const int64_t R0 = srow[s0], R1 = srow[s1];
+            int32_t at[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                at[i] = nearest_boundary(srow, s0, s1, R0 + (R1 - R0) * (i_lo + i) / ns);
+            t.st_lo = reinterpret_cast<const uint32_t*>(a.streams + B->stream + srow[at[0]]);
+            t.st_hi = reinterpret_cast<const uint32_t*>(a.streams + B->stream + srow[at[1]]);
+            t.g_lo = (int32_t)((srow[at[1]] - srow[at[0]]) / kRows);
+            t.g_hi = (int32_t)((srow[at[2]] - srow[at[1]]) / kRows);
+            t.g_max = __reduce_max_sync(kFull, max(t.g_lo, t.g_hi));
+            t.s_lo = at[0];
+            t.s_hi = at[1];
+            if (T.npass > 1 && (int64_t)t.g_max * kRows > (piped ? T.rows : a.bnd_stride)) {
+                if (lane == 0) atomicExch(a.err, 1);  // boundary buffer too small: refuse
+                break;
+            }
+            for (int pass = T.pass; pass < T.pass_end; ++pass) {
+                t.pass = pass;
+                t.done_in = piped && pass > 0 ? a.progress + ti - 1 : nullptr;
+                t.done_out = piped && pass + 1 < T.npass ? a.progress + ti : nullptr;
+                __syncwarp();
+                build_profile(a.db + qoff, m, (int64_t)pass * seg * T.R, T.R, seg, s_mat,
+                              B->swap ? 1 : MS, B->swap ? MS : 1, smem + warp * kSingleSmem);
+                if (two16) {
+                    switch (T.R) {
 #define CM_MODE 3
 #include "sw16_inst.cuh"
 #define CM_CASE(r) case r: single_dp<r, 16>(a, t); break;
-                    CM_R_CASES(CM_CASE)
+                        CM_R_CASES(CM_CASE)
 #undef CM_CASE
 #undef CM_MODE
-                }
-            } else {
-                switch (T.R) {
+                    }
+                } else {
+                    switch (T.R) {
 #define CM_MODE 1
 #include "sw16_inst.cuh"
 #define CM_CASE(r) case r: single_dp<r, 32>(a, t); break;
-                    CM_R_CASES(CM_CASE)
+                        CM_R_CASES(CM_CASE)
 #undef CM_CASE
 #undef CM_MODE
+                    }
                 }
             }
         }

@@ -1,0 +1,130 @@
+// The host harness of api_mock.cpp with the launchers that the library itself always has: the lone
+// queries of a plan in one launch of units, and its query pairs in one launch where that is the
+// rule.  The mocks compute the same fake scores and check what the kernels rely on: tickets and
+// progress words zeroed, the units of a task complete and in order, the boundary columns of
+// pipelined tasks apart and long enough, every stream of a piece of a unit within its slot, the
+// profiles of a merged launch within its shared memory.  A launch of one tile gets query pairs
+// only, as the kernel's.
+#include "ctx.h"
+
+#define launch_sw16 tile_launch
+#define main api_mock_main
+#include "api_mock.cpp"
+#undef main
+#undef launch_sw16
+
+namespace {
+
+SwArgs one_task(const SwArgs& a, const SwTask* t, int32_t* ticket)
+{
+    SwArgs b = a;
+    b.tasks = t;
+    b.ntasks = 1;
+    b.task_counter = ticket;
+    *ticket = 0;
+    return b;
+}
+
+// rows of the longest stream of subjects [s0, s1) split n ways
+int64_t longest_split(const int64_t* srow, int32_t s0, int32_t s1, int n)
+{
+    int64_t longest = 0;
+    for (int i = 0; i < n; ++i) {
+        const int64_t rows = srow[s1] - srow[s0];
+        const int32_t lo = nearest_boundary(srow, s0, s1, srow[s0] + rows * i / n);
+        const int32_t hi = nearest_boundary(srow, s0, s1, srow[s0] + rows * (i + 1) / n);
+        longest = std::max(longest, srow[hi] - srow[lo]);
+    }
+    return longest;
+}
+
+const char* unit_fault(const SwArgs& a, const SwUnit* units, int32_t t, int32_t first)
+{
+    const SwUnit& u = units[t];
+    const SwBlock& B = a.blocks[u.block];
+    const int64_t* srow = a.srows + B.srow;
+    const TileChoice tc = choose_tile(len_of(a.ids[B.a_ids + u.k]), false);
+    if (u.mode != tc.mode || u.R != tc.R || u.npass != tc.npass) return "unit of another tile";
+    if (u.s1 <= u.s0) return "unit without subjects";
+    const int ns = u.mode == kModeTwo16 ? 4 : 2;
+    if (u.bnd_row < 0) {
+        if (u.pass != 0 || u.pass_end != u.npass) return "unit of some passes without its column";
+        for (int32_t s0 = u.s0, s1; u.npass > 1 && s0 < u.s1; s0 = s1) {
+            s1 = piece_end(srow, s0, u.s1, a.bnd_stride);
+            if (s1 <= s0 || s1 > u.s1) return "piece out of its unit";
+            if (longest_split(srow, s0, s1, ns) > a.bnd_stride) return "stream longer than its slot";
+        }
+        return nullptr;
+    }
+    if (u.pass_end != u.pass + 1 || u.npass < 2) return "pipelined unit of several passes";
+    if (longest_split(srow, u.s0, u.s1, ns) > u.rows) return "boundary column too short";
+    if (u.pass > 0) {
+        const SwUnit& v = units[t - 1];
+        if (t == first || v.pass + 1 != u.pass || v.block != u.block || v.k != u.k || v.s0 != u.s0 ||
+            v.s1 != u.s1 || v.bnd_row != u.bnd_row)
+            return "pass that does not follow the one before it";
+    }
+    return nullptr;
+}
+
+}  // namespace
+
+namespace cm {
+
+cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st)
+{
+    if (mode != kModePair && mode != kModeSeg16) return cudaErrorInvalidValue;
+    return tile_launch(R, W, mode, grid, a, st);
+}
+
+cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaStream_t st)
+{
+    if (grid < 1 || W != 16) return cudaErrorInvalidValue;
+    if (*a.task_counter != 0) { contract_error(a, "task ticket not zeroed"); return cudaSuccess; }
+    for (int32_t i = 0; i < a.ntasks; ++i) {
+        const SwTask& t = a.tasks[i];
+        if (sw16_pair_smem(t.R, t.mode) > smem) { contract_error(a, "profile too large"); return cudaSuccess; }
+        int32_t ticket;
+        const cudaError_t e = launch_sw16(t.R, W, t.mode, grid, one_task(a, &t, &ticket), st);
+        if (e != cudaSuccess) return e;
+    }
+    *a.task_counter = a.ntasks;
+    return cudaSuccess;
+}
+
+cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_t st)
+{
+    if (grid < 1 || warps < 1 || warps > kSingleWarps) return cudaErrorInvalidValue;
+    const int32_t n = a.ranges[grid];
+    for (int r = 0; r < grid; ++r)
+        if (a.task_counter[r] != 0 || a.ranges[r + 1] < a.ranges[r]) {
+            contract_error(a, "ticket not zeroed, or ranges not in order");
+            return cudaSuccess;
+        }
+    int64_t columns = 0;                           // end of the boundary columns so far
+    for (int32_t t = 0; t < n; ++t) {
+        const SwUnit& u = a.units[t];
+        const char* fault = a.progress[t] != 0 ? "progress not zeroed" : unit_fault(a, a.units, t, 0);
+        if (!fault && u.bnd_row >= 0 && u.pass == 0) {
+            if (u.bnd_row < columns) fault = "boundary columns overlap";
+            columns = u.bnd_row + u.rows;
+        }
+        if (!fault && u.bnd_row >= 0 && u.pass + 1 < u.npass &&
+            (t + 1 == n || a.units[t + 1].pass != u.pass + 1))
+            fault = "task without its last pass";
+        if (fault) { contract_error(a, fault); return cudaSuccess; }
+        if (u.pass > 0) continue;                  // a task's scores, once
+        SwTask k{u.block, u.k, u.s0, u.s1, 1, 0, u.mode, u.R};
+        k.npass = u.npass;
+        int32_t ticket;
+        SwArgs b = one_task(a, &k, &ticket);
+        b.bnd_stride = INT64_MAX;                  // (its streams are checked above)
+        const cudaError_t e = tile_launch(u.R, 4, u.mode, grid, b, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace cm
+
+int main() { return api_mock_main(); }

@@ -1,0 +1,46 @@
+"""The host runtime with every launcher of the library (tests/launch_mock.cpp): the sessions of
+test_api_host.py on the launch of lone queries and the merged launch of query pairs, and plans
+whose boundary slots and unit ranges are where they can go wrong."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import test_api_host as api
+
+
+@pytest.fixture(scope="module")
+def exe(tmp_path_factory):
+    inc = api._cuda_include()
+    if shutil.which("g++") is None or inc is None:
+        pytest.skip("no host C++ compiler or CUDA headers")
+    path = str(tmp_path_factory.mktemp("launch") / "launch_mock")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", api.CSRC, "-I", inc, "-I",
+                    api.HERE, "-x", "c++", os.path.join(api.CSRC, "api.cu"), "-x", "c++",
+                    os.path.join(api.CSRC, "cluster_merge.cu"), "-x", "c++",
+                    os.path.join(api.HERE, "launch_mock.cpp"), "-o", path], check=True)
+    return path
+
+
+@pytest.mark.parametrize("session", [api.test_score_batch_cells_and_rerun, api.test_allpairs_parts,
+                                     api.test_cluster_merge_plain_ranked_and_batched])
+def test_sessions_on_every_launcher(exe, session):
+    session(exe)
+
+
+def test_ranked_lists_with_a_run_of_long_subjects(exe):
+    """A learned ClusterMerge whose lists, cut by count, put a run of long subjects, many times
+    the mean, into one task of a lone query of several passes: its streams are longer than a
+    boundary slot and the task runs in pieces."""
+    rng = np.random.default_rng(3)
+    short, long = (lambda n: rng.integers(40, 60, size=n)), (lambda n: rng.integers(1900, 2000, size=n))
+    L = np.concatenate([long(10), short(246), short(206), long(50)])
+    H = api.Harness(exe)
+    H.add("seqs %d %s" % (len(L), " ".join(map(str, L))), None)
+    H.add("sym 1", None)
+    H.add("sparse 1", None)
+    H.add("tuning 16 256", None)
+    H.add("cm 300 338 15 1 0", api._expect_cm(api._oracle_cm(L, 300, 338, 15, 1, 0, True)))
+    H.run()
