@@ -339,9 +339,8 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     a.nege2 = (uint32_t)(uint16_t)-P.ge * 0x10001u;
     a.sat_thr = (flags & CM_FORCE_INT32) ? -1 : P.sat_thr;   // -1: every pair goes to int32
 
-    // Launches.  All single-query tasks run in one launch, each CTA a contiguous range of them
-    // of an equal share of the cost: first the tasks of several passes, then tile by tile (the
-    // plan's order).  The query pairs of a plan that does not fill the chip tile by tile run in
+    // Launches.  All single-query tasks run in one launch, each CTA on a contiguous range of them
+    // (cut_ranges): first the tasks of several passes, then tile by tile (the plan's order).  The query pairs of a plan that does not fill the chip tile by tile run in
     // one launch too (with 16-warp CTAs, one per SM); those of a large plan, or of narrower CTAs,
     // in a persistent launch per (register tile, mode) bin.  (Builds without the launchers of
     // several tiles get a launch per bin.)
@@ -367,7 +366,6 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
             std::stable_partition(idx.begin(), idx.end(),
                                   [&](size_t x) { return plan.tasks[x].npass > 1; });
             std::vector<double> cost;
-            double total = 0;
             for (size_t i : idx) {
                 const SwTask& t = plan.tasks[i];
                 SwUnit u{t.block, t.k, t.s0, t.s1, t.npass, 0, t.npass, t.mode, t.R, 0, -1};
@@ -391,28 +389,22 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
                     if (piped) { u.pass = p; u.pass_end = p + 1; }
                     units.push_back(u);
                     cost.push_back(steps * t.R * (t.npass / n));
-                    total += cost.back();
                 }
             }
             const int64_t nu = (int64_t)units.size();
             if (nu >= INT32_MAX) return fail(c, CM_ERR_ARG, "too many tasks");
             const int grid = (int)std::min<int64_t>(nu, c->num_sms);
-            std::vector<int32_t> ranges(1, 0);
-            double sum = 0;
-            for (int64_t t = 0; t < nu; ++t) {
-                // CTA b ends at the first unit that reaches its share, leaving one for the others
-                sum += cost[t];
-                const int64_t b = (int64_t)ranges.size();
-                if (b < grid && (sum * grid >= total * b || nu - t - 1 == grid - b))
-                    ranges.push_back((int32_t)t + 1);
-            }
-            ranges.push_back((int32_t)nu);
+            std::vector<int32_t> ranges, homes;
+            cut_ranges(units, cost, grid, ranges, homes);
+            const int64_t nr = (int64_t)ranges.size() - 1;
+            ranges.insert(ranges.end(), homes.begin(), homes.end());
             ENSURE(B_UNITS, nu, d_units);
-            ENSURE(B_RANGE, 2 * grid + 1 + nu, d_ranges);
-            d_tickets = d_ranges + grid + 1;
+            ENSURE(B_RANGE, (int64_t)ranges.size() + nr + nu, d_ranges);
+            d_tickets = d_ranges + ranges.size();
             if ((r = copy_in(c, d_units, units.data(), units.size() * sizeof(SwUnit), false))) return r;
             if ((r = copy_in(c, d_ranges, ranges.data(), ranges.size() * sizeof(int32_t), false))) return r;
-            CUDA_TRY(cudaMemsetAsync(d_tickets, 0, (grid + nu) * sizeof(int32_t), st));
+            CUDA_TRY(cudaMemsetAsync(d_tickets, 0, (nr + nu) * sizeof(int32_t), st));
+            a.nranges = (int32_t)nr;
             const int warps = (int)std::min<int64_t>(kSingleWarps, (nu + grid - 1) / grid);
             launches.push_back({0, kModeTwo, grid, warps, 0, n_single, true, 0});
             // the plan's remaining tasks, in its order
@@ -495,7 +487,8 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         a.bnd = d_bnd + piped_rows + (side ? slots[0] : 0) * stride;
         a.units = d_units;
         a.ranges = d_ranges;
-        a.progress = L.single ? d_tickets + L.grid : nullptr;
+        a.homes = d_ranges + a.nranges + 1;
+        a.progress = L.single ? d_tickets + a.nranges : nullptr;
         a.piped = d_bnd;
         const cudaStream_t ls = side ? c->aux : st;
         le = L.single    ? launch_sw16_single(L.grid, L.warps_per_cta, a, ls)

@@ -116,7 +116,9 @@ struct SwArgs {
     int32_t ntasks;
     int32_t* task_counter;      // zeroed before launch
     const struct SwUnit* units; // single-query launch: its work units (instead of tasks)
-    const int32_t* ranges;      // ... first unit of each CTA (grid + 1)
+    const int32_t* ranges;      // ... first unit of each range (nranges + 1)
+    const int32_t* homes;       // ... the range each CTA starts with
+    int32_t nranges;
     int32_t* progress;          // ... boundary row groups written by each unit (zeroed)
     uint2* piped;               // ... boundary columns of the pipelined units
     const CellUnit* cell_units; // int32 launch: its units (null: the huge-score kernel)
@@ -224,8 +226,8 @@ cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaS
 cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaStream_t st)
     __attribute__((weak));
 // Every single-query task (kModeTwo, kModeTwo16; any tile width) in one launch of `grid` CTAs of
-// `warps` warps, a unit per warp at a time; CTA b owns the units [ranges[b], ranges[b + 1]),
-// task_counter[b] is its ticket.  Slots of bnd_stride rows for the units of all passes are
+// `warps` warps, a unit per warp at a time; range r holds the units [ranges[r], ranges[r + 1]),
+// task_counter[r] is its ticket.  Slots of bnd_stride rows for the units of all passes are
 // at bnd, one per warp.  Weak: a build with its own launch_sw16 and without this gets a launch
 // per bin.
 constexpr int kSingleWarps = 12;       // one CTA per SM: shared memory of the profiles

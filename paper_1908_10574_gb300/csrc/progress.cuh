@@ -1,8 +1,8 @@
 // Progress of a column pass over its rows, in a word of global memory: a pass of one warp writes
 // its boundary column row group by row group and publishes how many are written; the warp of
 // the next pass waits until the groups it is about to read are there.  A wait only ever points
-// at a pass whose warp is running (it took its unit from the queue earlier), so it ends; it is
-// bounded all the same.
+// at a pass whose warp is running: the passes of a task are handed out in order by one ticket.  So
+// it ends, whichever other CTAs are resident; it is bounded all the same.
 #pragma once
 #include <cstdint>
 

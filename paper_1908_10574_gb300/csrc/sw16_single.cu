@@ -8,17 +8,18 @@
 //     warp instead of a CTA whose other warps idle, and one launch takes the tasks of every
 //     register tile (the tile is a field of the task, the tile's code a function call): no
 //     launch per tile, no tail per launch.
-//   * The tasks come tile by tile, and a CTA (one per SM) owns a contiguous range of them of an
-//     equal share of the cost, so its warps run the same code: a tile's loop is 5-10 KB of
+//   * The tasks come tile by tile, and a CTA (one per SM) starts on a contiguous range of them of
+//     an equal share of the cost, so its warps run the same code: a tile's loop is 5-10 KB of
 //     instructions, and twelve warps on as many tiles miss the instruction cache (50,000
 //     pairs: 24 ms, 25 of 28 stall cycles per issue waiting for instructions).  Warps that
 //     find their CTA's range empty take from the others'.
 //   * The column passes of a long query (above 512 residues) are units of their own, taken by
 //     different warps: pass p trails pass p - 1 by 32 row groups over the boundary column in
 //     global memory, so a long query against long subjects is a pipeline, not one warp's
-//     serial chain (24 pairs of 10,000 residues: 53 ms as chains).  A unit's predecessor was
-//     taken before it, so its warp is running and waits only on passes before its own: the
-//     waits end.  Each is bounded all the same.
+//     serial chain (24 pairs of 10,000 residues: 53 ms as chains).  A task's units lie in one
+//     range, whose ticket hands them out in order: a unit's predecessor was taken before it, so
+//     its warp is running and waits only on passes before its own.  So the waits end, after the
+//     steps by which the passes trail one another.  Each is bounded all the same.
 //   * The profile holds plain matrix scores as bytes (any int8 matrix fits; pads are -128),
 //     four columns per word: 16 KB for 512 columns, so 12 warps fit an SM.  The packed score
 //     of a column for the two streams' residues is one byte permute with sign extension of
@@ -250,7 +251,7 @@ __device__ __forceinline__ void build_profile(const uint8_t* q, int64_t m, int64
     __syncwarp();
 }
 
-// A warp runs tasks of its CTA's range until it is empty, then of the ranges after it.
+// A warp runs units of its CTA's first range until it is empty, then of the ranges after it.
 // kModeTwo: the task's rows split into two streams at subject boundaries, over 32 lanes, in
 // passes of 32 R columns whose boundary column goes through the warp's slot of `bnd`;
 // kModeTwo16: four streams, two per 16-lane segment.
@@ -268,8 +269,9 @@ sw16_single_kernel(const __grid_constant__ SwArgs a)
     __syncthreads();
     uint4* bnd = reinterpret_cast<uint4*>(
         a.bnd + ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * a.bnd_stride);
-    for (int visited = 0; visited < (int)gridDim.x;) {
-        const int range = (blockIdx.x + visited) % gridDim.x;
+    const int home = a.homes[blockIdx.x];
+    for (int visited = 0; visited < a.nranges;) {
+        const int range = (home + visited) % a.nranges;
         int ti = 0;
         if (lane == 0) ti = a.ranges[range] + atomicAdd(a.task_counter + range, 1);
         ti = __shfl_sync(kFull, ti, 0);

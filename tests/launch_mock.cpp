@@ -3,8 +3,8 @@
 // rule.  The mocks compute the same fake scores and check what the kernels rely on: tickets and
 // progress words zeroed, the units of a task complete and in order, the boundary columns of
 // pipelined tasks apart and long enough, every stream of a piece of a unit within its slot, the
-// profiles of a merged launch within its shared memory.  A launch of one tile gets query pairs
-// only, as the kernel's.
+// profiles of a merged launch within its shared memory, a task's units in one range (the first unit
+// of a range waits for nobody).  A launch of one tile gets query pairs only, as the kernel's.
 #include "ctx.h"
 
 #define launch_sw16 tile_launch
@@ -95,16 +95,25 @@ cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaSt
 cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_t st)
 {
     if (grid < 1 || warps < 1 || warps > kSingleWarps) return cudaErrorInvalidValue;
-    const int32_t n = a.ranges[grid];
-    for (int r = 0; r < grid; ++r)
-        if (a.task_counter[r] != 0 || a.ranges[r + 1] < a.ranges[r]) {
-            contract_error(a, "ticket not zeroed, or ranges not in order");
+    const int32_t n = a.ranges[a.nranges];
+    if (a.nranges < 1 || a.nranges > grid || a.ranges[0] != 0) { contract_error(a, "ranges"); return cudaSuccess; }
+    std::vector<int32_t> range_of((size_t)n, 0);
+    std::vector<char> home((size_t)a.nranges, 0);
+    for (int b = 0; b < grid; ++b) {
+        if (a.homes[b] < 0 || a.homes[b] >= a.nranges) { contract_error(a, "home"); return cudaSuccess; }
+        home[a.homes[b]] = 1;
+    }
+    for (int r = 0; r < a.nranges; ++r) {
+        if (a.task_counter[r] != 0 || a.ranges[r + 1] <= a.ranges[r] || !home[r]) {
+            contract_error(a, "ticket not zeroed, or a range empty or without a CTA");
             return cudaSuccess;
         }
+        for (int32_t t = a.ranges[r]; t < a.ranges[r + 1]; ++t) range_of[t] = a.ranges[r];
+    }
     int64_t columns = 0;                           // end of the boundary columns so far
     for (int32_t t = 0; t < n; ++t) {
         const SwUnit& u = a.units[t];
-        const char* fault = a.progress[t] != 0 ? "progress not zeroed" : unit_fault(a, a.units, t, 0);
+        const char* fault = a.progress[t] != 0 ? "progress not zeroed" : unit_fault(a, a.units, t, range_of[t]);
         if (!fault && u.bnd_row >= 0 && u.pass == 0) {
             if (u.bnd_row < columns) fault = "boundary columns overlap";
             columns = u.bnd_row + u.rows;

@@ -44,3 +44,19 @@ def test_ranked_lists_with_a_run_of_long_subjects(exe):
     H.add("tuning 16 256", None)
     H.add("cm 300 338 15 1 0", api._expect_cm(api._oracle_cm(L, 300, 338, 15, 1, 0, True)))
     H.run()
+
+
+def test_pipelined_tasks_stay_in_one_range(exe):
+    """Lists of a few queries of many passes: an equal share of the cost ends inside a task, whose
+    passes have to stay with one ticket all the same."""
+    rng = np.random.default_rng(8)
+    H = api.Harness(exe)
+    for k, q in ((1, 9000), (3, 6000), (7, 2000), (40, 700)):
+        L = np.concatenate([rng.integers(q, q + 500, size=k), rng.integers(100, 400, size=5)])
+        pairs = [(a, int(rng.integers(0, k + 5))) for a in range(k) for _ in range(6)]
+        flat = " ".join("%d %d" % p for p in pairs)
+        H.add("seqs %d %s" % (len(L), " ".join(map(str, L))), None)
+        H.add("sym 0", None)
+        H.add("score 0 %d %s" % (len(pairs), flat),
+              api._expect_values("score", [api._score(a, b, L, False) for a, b in pairs]))
+    H.run()
