@@ -27,8 +27,8 @@ def test_ranked_merge_of_a_run_of_long_subjects():
 
     seqs = [long(1990), long(1950)] + [synth.random_seq(rng, int(n)) for n in rng.integers(40, 60, 126)]
     seqs[100] = seqs[101].copy()                   # they merge: an odd number of queries, the longest alone
-    seqs += [synth.random_seq(rng, int(n)) for n in rng.integers(40, 60, 98)]
-    seqs += [long(int(n)) for n in rng.integers(1900, 2000, 30)]
+    seqs += [synth.random_seq(rng, int(n)) for n in rng.integers(40, 60, 108)]
+    seqs += [long(int(n)) for n in rng.integers(1900, 2000, 20)]
     ss = synth.SeqSet.from_list(seqs)
     n = len(ss)
     _, scores = oracle.all_pairs(ss.seqs, ss.offsets, S62, 11, 1, T=100)
