@@ -225,15 +225,65 @@ batch_rows_kernel(const uint8_t* __restrict__ db, const int64_t* __restrict__ of
 // of a sequence: the column sum less the 4 - t last rows (t < 4) or the t - 4 first ones.  1,152
 // products per channel and sequence instead of per row: 65 us for 4,000 sequences, where the
 // layer over their 1.7M rows took 361 us and the second one wrote 433 MB for it.
-// One block per kPoolSeqs sequences: the S_t in shared memory (fixed-point differences, exact),
-// each thread two channels of a quarter of K for all of them, FP32.
+// One block per kPoolSeqs sequences: the S_t, times inv_pow2_len, in shared memory (integer
+// differences; what is rounded before them is the FP32 sum of up to 32 rows that the second
+// layer's epilogue adds at once), each thread two channels of a quarter of K for all of them, FP32.
 constexpr int kPoolSeqs = 8;
+
+// Scale of the second layer's column sums: 2^s with B 2^s in [2^58, 2^59), B a bound on the layer's
+// activations for any sequence,
+//   B = max_n |b2[n]| + sum |W2| z1,   z1[n] = |b1[n]| + sum |W1| max_code |E|,
+// so that activations, up to twice B with their own rounding, leave three bits of 64.  A power of
+// two, so scaling rounds nothing.  One block over 370 KB of weights, 10 us, in the first
+// embedding call after the weights change.
+__global__ void __launch_bounds__(1024)
+sum_scale_kernel(const bf16* __restrict__ E, const bf16* __restrict__ W1, const float* __restrict__ b1,
+                 const bf16* __restrict__ W2, const float* __restrict__ b2, float* __restrict__ scale)
+{
+    __shared__ float x0[kEmb], z1[kCh], top[kCh];
+    const int n = threadIdx.x >> 3, part = threadIdx.x & 7;      // eight threads a channel
+    if (threadIdx.x < kEmb) {
+        float m = 0.f;
+        for (int code = 0; code < 20; ++code) m = fmaxf(m, fabsf(__bfloat162float(E[code * kEmb + threadIdx.x])));
+        x0[threadIdx.x] = m;
+    }
+    __syncthreads();
+    // |bias[n]| + sum over k of |W[n][k]| x[k mod cin], eight values a load
+    auto bound = [&](const bf16* W, int cin, const float* x, float bias) {
+        float t = 0.f;
+        for (int k = part * 8; k < kTaps * cin; k += 64) {
+            const uint4 w = *reinterpret_cast<const uint4*>(W + (int64_t)n * kTaps * cin + k);
+            const __nv_bfloat162* v = reinterpret_cast<const __nv_bfloat162*>(&w);
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                t += fabsf(__bfloat162float(v[h].x)) * x[(k + 2 * h) % cin] +
+                     fabsf(__bfloat162float(v[h].y)) * x[(k + 2 * h + 1) % cin];
+        }
+        for (int d = 4; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+        return t + fabsf(bias);
+    };
+    const float t1 = bound(W1, kEmb, x0, b1[n]);
+    if (part == 0) z1[n] = t1;
+    __syncthreads();
+    const float t2 = bound(W2, kCh, z1, b2[n]);
+    if (part == 0) top[n] = t2;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    // the largest as bits, which order as the values do: infinities and NaN above all
+    uint32_t m = 0;
+    for (int i = threadIdx.x; i < kCh; i += 32) m = max(m, __float_as_uint(top[i]) & 0x7fffffffu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    const int e = m < 0x00800000u ? -126 : (int)(m >> 23) - 127;  // B < 2^(e + 1)
+    if (threadIdx.x == 0) *scale = scalbnf(1.f, min(58 - e, 126));
+}
 
 __global__ void __launch_bounds__(256)
 pool_linear_kernel(const unsigned long long* __restrict__ sums, const bf16* __restrict__ edge,
                    const int32_t* __restrict__ slen, int64_t ns, const bf16* __restrict__ W3T,
-                   const float* __restrict__ b3, float* __restrict__ V)
+                   const float* __restrict__ b3, const float* __restrict__ sum_scale,
+                   float* __restrict__ V)
 {
+    const float scale = *sum_scale;
     __shared__ __align__(16) float S[kTaps * kCh][kPoolSeqs];
     __shared__ float red[3][kPoolSeqs][kCh];
     const int64_t s0 = (int64_t)blockIdx.x * kPoolSeqs;
@@ -243,9 +293,9 @@ pool_linear_kernel(const unsigned long long* __restrict__ sums, const bf16* __re
         const int len = s < ns ? slen[s] : 0;
         const long long total = len > 0 ? (long long)sums[s * kCh + c] : 0;
         auto row = [&](int k) {                    // k: 0..3 from the start, 4..7 from the end
-            return to_fixed(__bfloat162float(edge[(s * 8 + k) * kCh + c]));
+            return to_fixed(__bfloat162float(edge[(s * 8 + k) * kCh + c]), sum_unit(scale, len));
         };
-        auto put = [&](int t, long long x) { S[t * kCh + c][q] = (float)x * (float)(1.0 / kPoolScale); };
+        auto put = [&](int t, long long x) { S[t * kCh + c][q] = (float)x * (1.f / scale); };
         put(4, total);
         long long lo = total, hi = total;
         for (int d = 1; d <= 4; ++d) {
@@ -301,7 +351,8 @@ pool_linear_kernel(const unsigned long long* __restrict__ sums, const bf16* __re
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float t = acc[q][h] + red[0][q][n + h] + red[1][q][n + h] + red[2][q][n + h];
-            V[(s0 + q) * kCh + n + h] = len > 0 ? t / (float)len + b3[n + h] : 0.f;
+            // (S holds the sums times inv_pow2_len: a division by a value in (1/2, 1])
+            V[(s0 + q) * kCh + n + h] = len > 0 ? t / ((float)len * inv_pow2_len(len)) + b3[n + h] : 0.f;
         }
     }
 }
@@ -467,13 +518,14 @@ struct Ranker {
     int32_t* tc_err = nullptr;                  // error word of the tensor-core kernels
     int64_t step = 0;
     bool ready = false;
+    bool scaled = false;                        // A_SCALE is of the present weights
     // activation buffers (grown on demand)
     DevBuf act[24];
 };
 
 enum ActId { A_CODES, A_ROWSEQ, A_X0, A_Z1, A_Z2, A_DZ, A_DY2, A_PART, A_V, A_DV,
              A_SEQ, A_PIDX, A_Y, A_LOGIT, A_EP_SID, A_EP_SROW, A_EP_SLEN, A_EP_PIDX, A_EP_Y,
-             A_V64, A_EDGE };
+             A_V64, A_EDGE, A_SCALE };
 
 namespace {
 
@@ -555,6 +607,7 @@ int get_ranker(cm_ctx* c, Ranker** out)
 int refresh_bf16(cm_ctx* c, Ranker* K)
 {
     const cudaStream_t st = c->stream;
+    K->scaled = false;
     cast_kernel<<<blocks_for(20 * kEmb, 256), 256, 0, st>>>(K->params + kOffE, K->E, 20 * kEmb);
     cast_weights_kernel<<<blocks_for((int64_t)kTaps * kEmb * kCh, 256), 256, 0, st>>>(
         K->params + kOffW1, kEmb, K->W1, K->W1T);
@@ -625,11 +678,12 @@ int check_tc(cm_ctx* c, Ranker* K)
 }
 
 // forward over a batch whose layout (sequence ids, first rows, lengths; R rows) is on the
-// device; leaves the pooled vectors V on the device, and with `train` the activations X0, Z1 and
-// Z2 and the row metadata for the backward pass
+// device; leaves the pooled vectors V on the device.  Inference has `scale` (sum_scale_kernel);
+// training, without it, also leaves the activations X0, Z1 and Z2 and the row metadata for the
+// backward pass
 int forward_dev(cm_ctx* c, const Prepared& P, Ranker* K, const int32_t* d_sid,
-                const int64_t* d_srow, const int32_t* d_slen, int64_t ns, int64_t R, bool train,
-                float** V_out)
+                const int64_t* d_srow, const int32_t* d_slen, int64_t ns, int64_t R,
+                const float* scale, float** V_out)
 {
     const cudaStream_t st = c->stream;
     uint8_t* codes; int32_t* rowseq; bf16 *X0, *Z1; float* V; unsigned long long* V64;
@@ -653,15 +707,16 @@ int forward_dev(cm_ctx* c, const Prepared& P, Ranker* K, const int32_t* d_sid,
     ep.bias = K->params + kOffB2;
     ep.slen = d_slen;
     ep.acc64 = V64;
-    if (!train) {
+    if (scale) {
         bf16* edge;
         AENSURE(A_EDGE, ns * 8 * kCh * 2, edge);
         ep.out = nullptr;
         ep.srow = d_srow;
         ep.edge = edge;
+        ep.scale = scale;
         if ((r = conv_tc<kCh, kCh, kEpiSum>(c, K, Z1, R, K->W2, ep))) return r;
         pool_linear_kernel<<<blocks_for(ns, kPoolSeqs), 256, 0, st>>>(V64, edge, d_slen, ns, K->W3T,
-                                                                      K->params + kOffB3, V);
+                                                                      K->params + kOffB3, scale, V);
     } else {
         bf16* Z2;
         AENSURE(A_Z2, R * kCh * 2, Z2);
@@ -680,7 +735,7 @@ int forward_dev(cm_ctx* c, const Prepared& P, Ranker* K, const int32_t* d_sid,
 }
 
 // inference over a batch laid out on the host
-int forward(cm_ctx* c, const Prepared& P, Ranker* K, const Batch& B, float** V_out)
+int forward(cm_ctx* c, const Prepared& P, Ranker* K, const Batch& B, const float* scale, float** V_out)
 {
     const int64_t ns = (int64_t)B.sid.size();
     int32_t* seqinfo;
@@ -692,7 +747,7 @@ int forward(cm_ctx* c, const Prepared& P, Ranker* K, const Batch& B, float** V_o
     if ((r = copy_in(c, d_sid, B.sid.data(), ns * 4, false))) return r;
     if ((r = copy_in(c, d_srow, B.srow.data(), ns * 8, false))) return r;
     if ((r = copy_in(c, d_slen, B.slen.data(), ns * 4, false))) return r;
-    return forward_dev(c, P, K, d_sid, d_srow, d_slen, ns, B.R, false, V_out);
+    return forward_dev(c, P, K, d_sid, d_srow, d_slen, ns, B.R, scale, V_out);
 }
 
 // weight gradient of a conv layer on the tensor cores: the rows are cut into chunks so that
@@ -799,7 +854,7 @@ int loss_grad_packed(cm_ctx* c, const Prepared& P, Ranker* K, const Packed& B, c
     const int64_t R = B.rows[b];
     const int32_t* d_slen = D.slen + so;
     float* V;
-    int r = forward_dev(c, P, K, D.sid + so, D.srow + so, d_slen, ns, R, true, &V);
+    int r = forward_dev(c, P, K, D.sid + so, D.srow + so, d_slen, ns, R, nullptr, &V);
     if (r) return r;
     const int32_t* d_pidx = D.pidx + 2 * po;
     const float* d_y = D.y + po;
@@ -861,6 +916,15 @@ int ranker_embed_device(cm_ctx* c, const Prepared& P, const int32_t* ids, int64_
     int r = get_ranker(c, &K);
     if (r) return r;
     if (!K->ready) return fail(c, CM_ERR_ARG, "ranker has no parameters (init, train or load first)");
+    float* scale;
+    AENSURE(A_SCALE, sizeof(float), scale);
+    if (!K->scaled) {
+        sum_scale_kernel<<<1, 1024, 0, c->stream>>>(K->E, K->W1, K->params + kOffB1, K->W2,
+                                                    K->params + kOffB2, scale);
+        CUDA_TRY(cudaGetLastError());
+        c->stats.launches += 1;
+        K->scaled = true;
+    }
     const int64_t max_rows = (int64_t)1 << 22;   // activation budget per chunk
     int64_t i = 0;
     while (i < n) {
@@ -872,7 +936,7 @@ int ranker_embed_device(cm_ctx* c, const Prepared& P, const int32_t* ids, int64_
         Batch B;
         layout(P, ids + i, j - i, B);
         float* Vc;
-        if ((r = forward(c, P, K, B, &Vc))) return r;
+        if ((r = forward(c, P, K, B, scale, &Vc))) return r;
         CUDA_TRY(cudaMemcpyAsync(V + i * kCh, Vc, (j - i) * kCh * 4, cudaMemcpyDeviceToDevice,
                                  c->stream));
         i = j;
@@ -1111,6 +1175,7 @@ int cm_ranker_train(cm_ctx* c, const uint8_t* seqs, const int64_t* offsets, int3
     float loss = 0.f;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const Bf16Copies copies{K->E, K->W1, K->W1T, K->W2, K->W2T, K->W3, K->W3T};
+    K->scaled = false;
     int64_t total_steps = 0, t_step = 0;      // for CM_TRAIN_COSINE (batches per epoch are fixed)
     for (int ep = 0; ep < epochs; ++ep) {
         // the whole epoch's batches go to the device in one copy per array

@@ -31,9 +31,12 @@ namespace cm {
 //              pre-pooling activations are never stored).  The sums are kept in 64-bit fixed
 //              point (units of 2^-32) so that the atomic adds commute: v does not depend on
 //              the order in which CTAs finish, and neither do the ranker's logits.
-//   kEpiSum    colsum[seq] += bf16(relu(acc + bias)) over every real row, in fixed point as Pool;
-//              the rows within 4 of a sequence's ends also go to `edge`, the others nowhere (the
-//              linear third layer needs no more of the second one, see pool_linear_kernel)
+//   kEpiSum    colsum[seq] += bf16(relu(acc + bias)) over every real row, in 64-bit fixed point
+//              like Pool but in units of the weights' scale and the sequence's length (sum_unit),
+//              so that no sum of these activations can leave 64 bits or fall below the unit
+//              whatever the scale of the weights; the rows within 4 of a sequence's ends also go
+//              to `edge`, the others nowhere (the linear third layer needs no more of the second
+//              one, see pool_linear_kernel)
 //   kEpiGate   out = bf16(gate > 0 ? acc : 0), and colsum[n] += the column sums of those
 //              values (the bias gradient of the layer below)
 //   kEpiEmbed  dE[code][c] += acc for every real row (the embedding table's gradient; dX0 is
@@ -50,14 +53,27 @@ struct ConvEpi {
     __nv_bfloat16* edge;        // Sum: ns x 8 x NOUT, rows 0..3 from the start, 0..3 from the end
     const uint8_t* codes;       // Embed: residue code of every row
     float* acc;                 // Gate: column sums; Embed: dE (20 x NOUT)
-    unsigned long long* acc64;  // Pool: v, Sum: column sums (ns x NOUT) in units of 2^-32
+    unsigned long long* acc64;  // Pool: v in units of 2^-32, Sum: column sums (ns x NOUT)
+    const float* scale;         // Sum: units of an activation of 1 in a sequence of one row
 };
 
 constexpr double kPoolScale = 4294967296.0;   // 2^32: fixed-point unit of the pooled sums
 
 // v in fixed point: the scaling by a power of two is exact in float, so only the conversion
 // rounds (to nearest); no double-precision operation
-__device__ __forceinline__ long long to_fixed(float v) { return __float2ll_rn(v * (float)kPoolScale); }
+__device__ __forceinline__ long long to_fixed(float v, float unit = (float)kPoolScale)
+{
+    return __float2ll_rn(v * unit);
+}
+
+// 2^-k for the least k with 2^k >= len: with it a sum over a sequence's rows is no larger than the
+// largest of them
+__device__ __forceinline__ float inv_pow2_len(int len)
+{
+    return __int_as_float((127 - (len <= 1 ? 0 : 32 - __clz(len - 1))) << 23);
+}
+// fixed-point units of an activation of 1 in the column sums of a sequence of `len` rows
+__device__ __forceinline__ float sum_unit(float scale, int len) { return scale * inv_pow2_len(len); }
 
 namespace tc {
 
@@ -158,6 +174,7 @@ struct ConvCfg {
 struct EpiRow {
     int32_t seq;             // < 0: a gap row, or past the end
     float inv_len;           // Pool
+    float unit;              // Sum
     int edge_lo, edge_hi;    // Sum: distance to the sequence's first and last row
     int code;                // Embed
     bool binned;
@@ -165,7 +182,7 @@ struct EpiRow {
 };
 
 template <int NOUT, int EPI>
-__device__ __forceinline__ EpiRow epi_row(int64_t r, int64_t R, int j0, const ConvEpi& ep)
+__device__ __forceinline__ EpiRow epi_row(int64_t r, int64_t R, int j0, const ConvEpi& ep, float scale)
 {
     EpiRow e{};
     const bool in = r < R;
@@ -173,8 +190,10 @@ __device__ __forceinline__ EpiRow epi_row(int64_t r, int64_t R, int j0, const Co
     if (EPI == kEpiPool && e.seq >= 0) e.inv_len = 1.f / (float)ep.slen[e.seq];
     if (EPI == kEpiSum && e.seq >= 0) {
         const int64_t pos = r - ep.srow[e.seq];
+        const int len = ep.slen[e.seq];
         e.edge_lo = (int)min(pos, (int64_t)4);
-        e.edge_hi = (int)min((int64_t)ep.slen[e.seq] - 1 - pos, (int64_t)4);
+        e.edge_hi = (int)min((int64_t)len - 1 - pos, (int64_t)4);
+        e.unit = sum_unit(scale, len);
     }
     if (EPI == kEpiEmbed) {
         // rows of letters outside the 20 embedded ones (zero embedding) add nothing
@@ -214,10 +233,14 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
     // Pool, Sum: a warp whose real rows all belong to one sequence reduces its 32 rows first
     int32_t lead = -1;
     bool one_seq = false;
+    float unit = (float)kPoolScale;                // of that sequence
     if (EPI == kEpiPool || EPI == kEpiSum) {
         lead = __reduce_max_sync(0xffffffffu, e.seq);
         one_seq = __all_sync(0xffffffffu, e.seq < 0 || e.seq == lead);
+        // (positive floats order as their bits; gap rows have 0)
+        if (EPI == kEpiSum) unit = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(e.unit)));
     }
+    const float row_unit = EPI == kEpiSum ? e.unit : (float)kPoolScale;
 #pragma unroll 1
     for (int j = j0; j < j1; ++j) {
         float v[32];
@@ -278,7 +301,7 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
             if (one_seq) {
                 const float t = warp_colsum32(v, lane);
                 if (lead >= 0)
-                    atomicAdd(ep.acc64 + (int64_t)lead * NOUT + n0 + lane, (unsigned long long)to_fixed(t));
+                    atomicAdd(ep.acc64 + (int64_t)lead * NOUT + n0 + lane, (unsigned long long)to_fixed(t, unit));
             } else {
                 // the rows of each sequence, summed in fixed point (one atomic per column)
                 uint32_t left = __ballot_sync(0xffffffffu, real);
@@ -286,7 +309,7 @@ __device__ __forceinline__ void conv_epilogue(uint32_t tacc, int q, int lane, in
                     const int32_t seq = __shfl_sync(0xffffffffu, e.seq, __ffs(left) - 1);
                     long long w[32];
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) w[t] = e.seq == seq ? to_fixed(v[t]) : 0;
+                    for (int t = 0; t < 32; ++t) w[t] = e.seq == seq ? to_fixed(v[t], row_unit) : 0;
                     const long long t = warp_colsum32(w, lane);
                     atomicAdd(ep.acc64 + (int64_t)seq * NOUT + n0 + lane, (unsigned long long)t);
                     left &= ~__ballot_sync(0xffffffffu, e.seq == seq);
@@ -479,12 +502,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int j1 = kEpiActive == 8 ? (half + 1) * (NCH / 2) : NCH;
         float* emb = s_emb + (EPI == kEpiEmbed ? ew * (32 * 33 + 20 * NOUT) : 0);
         uint8_t* out = bring + S * C::STAGE_BYTES + (warp - 2) * (32 * 128);
+        const float scale = EPI == kEpiSum ? *ep.scale : 0.f;
         int i = group;
         for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < ntiles;
              tile += (int64_t)C::GROUPS * gridDim.x, i += C::GROUPS) {
             const int b = i & 1;
             const int64_t row0 = tile * kTcRows + q * 32;
-            const EpiRow er = epi_row<NOUT, EPI>(row0 + lane, R, j0, ep);
+            const EpiRow er = epi_row<NOUT, EPI>(row0 + lane, R, j0, ep, scale);
             const bool ok = mbar_wait(&tfull[b], (i / 2) & 1, err);
             if (!__all_sync(0xffffffffu, ok)) break;      // warp-uniform: tcgen05.ld is warp-wide
             fence_after_sync();
