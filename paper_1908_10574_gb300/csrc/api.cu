@@ -286,9 +286,10 @@ int rescore(cm_ctx* c, const Prepared& P, const SwArgs& a, std::vector<PairRef>&
 }  // namespace
 
 // ---- execution --------------------------------------------------------------------------
-int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64_t* d_omap,
+int run_plan(cm_ctx* c, const Prepared& P, Plan& plan_in, int32_t* out, const int64_t* d_omap,
              uint32_t flags)
 {
+    const Plan& plan = plan_in;                  // left as it is: the autotuner runs it again
     const cudaStream_t st = c->stream;
     const int W = c->W;
     // upload
@@ -340,10 +341,11 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     a.sat_thr = (flags & CM_FORCE_INT32) ? -1 : P.sat_thr;   // -1: every pair goes to int32
 
     // Launches.  All single-query tasks run in one launch, each CTA on a contiguous range of them
-    // (cut_ranges): first the tasks of several passes, then tile by tile (the plan's order).  The query pairs of a plan that does not fill the chip tile by tile run in
-    // one launch too (with 16-warp CTAs, one per SM); those of a large plan, or of narrower CTAs,
-    // in a persistent launch per (register tile, mode) bin.  (Builds without the launchers of
-    // several tiles get a launch per bin.)
+    // (cut_ranges): first the tasks of several passes, then tile by tile (the plan's order).  The
+    // query pairs of a plan that does not fill the chip tile by tile run in one launch too (with
+    // 16-warp CTAs, one per SM); those of a large plan, or of narrower CTAs, in a persistent launch
+    // per (register tile, mode) bin.  (Builds without the launchers of several tiles get a launch
+    // per bin.)
     struct Launch {
         int R, mode, grid, warps_per_cta;
         size_t i0, i1;
@@ -356,9 +358,9 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     int32_t *d_ranges = nullptr, *d_tickets = nullptr;
     SwUnit* d_units = nullptr;
     int64_t piped_rows = 0;
+    auto single = [](const SwTask& t) { return t.mode == kModeTwo || t.mode == kModeTwo16; };
     if (launch_sw16_single) {
         std::vector<size_t> idx;
-        auto single = [&](const SwTask& t) { return t.mode == kModeTwo || t.mode == kModeTwo16; };
         for (size_t i = 0; i < plan.tasks.size(); ++i)
             if (single(plan.tasks[i])) idx.push_back(i);
         n_single = idx.size();
@@ -407,40 +409,45 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
             a.nranges = (int32_t)nr;
             const int warps = (int)std::min<int64_t>(kSingleWarps, (nu + grid - 1) / grid);
             launches.push_back({0, kModeTwo, grid, warps, 0, n_single, true, 0});
-            // the plan's remaining tasks, in its order
-            size_t k = 0;
-            for (size_t i = 0; i < plan.tasks.size(); ++i)
-                if (!single(plan.tasks[i])) {
-                    plan.tasks[k] = plan.tasks[i];
-                    plan.task_R[k] = plan.task_R[i];
-                    plan.keys[k++] = plan.keys[i];
-                }
-            plan.tasks.resize(k);
-            plan.task_R.resize(k);
-            plan.keys.resize(k);
         }
+    }
+    // the plan's other tasks, bin by bin in its order, or copies of them in another list
+    const SwTask* tasks = plan.tasks.data();
+    const int* bin = plan.task_R.data();
+    size_t nt = plan.tasks.size();
+    std::vector<SwTask> own_tasks;
+    std::vector<int> own_bins;
+    std::vector<std::pair<int64_t, size_t>> order;   // (-cost, index in the plan)
+    if (n_single > 0) {
+        for (size_t i = 0; i < nt; ++i)
+            if (!single(plan.tasks[i])) {
+                own_tasks.push_back(plan.tasks[i]);
+                own_bins.push_back(plan.task_R[i]);
+                order.push_back({-plan.keys[i].first, i});
+            }
+        tasks = own_tasks.data();
+        bin = own_bins.data();
+        nt = own_tasks.size();
     }
     int pair_smem = 0;
     int bins = 0;                                 // the tasks come bin by bin
-    for (size_t i = 0; i < plan.tasks.size(); ++i)
-        bins += i == 0 || plan.task_R[i] != plan.task_R[i - 1];
-    const bool one_pairs = W == 16 && launch_sw16_pairs && !plan.tasks.empty() &&
-                           (double)plan.tasks.size() <= kMergedTasks * bins * c->num_sms;
+    for (size_t i = 0; i < nt; ++i) bins += i == 0 || bin[i] != bin[i - 1];
+    const bool one_pairs = W == 16 && launch_sw16_pairs && nt > 0 &&
+                           (double)nt <= kMergedTasks * bins * c->num_sms;
     if (one_pairs) {                              // longest first, whatever their tile
-        const size_t n = plan.tasks.size();
-        std::vector<std::pair<int64_t, size_t>> order(n);
-        for (size_t i = 0; i < n; ++i) order[i] = {-plan.keys[i].first, i};
+        if (n_single == 0)
+            for (size_t i = 0; i < nt; ++i) order.push_back({-plan.keys[i].first, i});
         std::sort(order.begin(), order.end());
-        std::vector<SwTask> t2(n);
-        for (size_t i = 0; i < n; ++i) t2[i] = plan.tasks[order[i].second];
-        plan.tasks.swap(t2);
-        for (const SwTask& t : plan.tasks) pair_smem = std::max(pair_smem, sw16_pair_smem(t.R, t.mode));
-        launches.push_back({0, kModePair, (int)std::min<int64_t>((int64_t)n, c->num_sms), W, 0, n, false, 0});
+        own_tasks.resize(nt);
+        for (size_t i = 0; i < nt; ++i) own_tasks[i] = plan.tasks[order[i].second];
+        tasks = own_tasks.data();
+        for (size_t i = 0; i < nt; ++i) pair_smem = std::max(pair_smem, sw16_pair_smem(tasks[i].R, tasks[i].mode));
+        launches.push_back({0, kModePair, (int)std::min<int64_t>((int64_t)nt, c->num_sms), W, 0, nt, false, 0});
     }
-    for (size_t i0 = one_pairs ? plan.tasks.size() : 0; i0 < plan.tasks.size();) {
-        const int key = plan.task_R[i0];
+    for (size_t i0 = one_pairs ? nt : 0; i0 < nt;) {
+        const int key = bin[i0];
         size_t i1 = i0;
-        while (i1 < plan.tasks.size() && plan.task_R[i1] == key) ++i1;
+        while (i1 < nt && bin[i1] == key) ++i1;
         const int64_t resident = (int64_t)c->num_sms * sw16_occupancy(c, key / 4, W, key % 4);
         launches.push_back({key / 4, key % 4, (int)std::min<int64_t>((int64_t)(i1 - i0), resident), W,
                             i0, i1, false, 0});
@@ -448,7 +455,7 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
     }
     if ((int)launches.size() > kTaskBins)
         return fail(c, CM_ERR_INTERNAL, "more launch bins than task tickets");
-    if ((r = copy_in(c, d_tasks, plan.tasks.data(), plan.tasks.size() * sizeof(SwTask), false))) return r;
+    if ((r = copy_in(c, d_tasks, tasks, nt * sizeof(SwTask), false))) return r;
 
     // boundary buffer of the tasks with several column passes (a slot per resident warp; even
     // strides, so the records of two rows stay 16-byte aligned).  Launches alternate between
@@ -461,7 +468,7 @@ int run_plan(cm_ctx* c, const Prepared& P, Plan& plan, int32_t* out, const int64
         if (L.single) {
             for (const SwUnit& u : units) passes = passes || u.pass_end - u.pass > 1;
         } else {
-            for (size_t i = L.i0; i < L.i1 && !passes; ++i) passes = plan.tasks[i].npass > 1;
+            for (size_t i = L.i0; i < L.i1 && !passes; ++i) passes = tasks[i].npass > 1;
         }
         L.warps = passes ? (int64_t)L.grid * L.warps_per_cta : 0;
         slots[(l + 1) & 1] = std::max(slots[(l + 1) & 1], L.warps);

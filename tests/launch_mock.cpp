@@ -8,12 +8,23 @@
 #include "ctx.h"
 
 #define launch_sw16 tile_launch
+#define launch_gather_stream gather_stream
 #define main api_mock_main
 #include "api_mock.cpp"
 #undef main
+#undef launch_gather_stream
 #undef launch_sw16
 
 namespace {
+
+std::vector<std::string> g_runs;                   // per plan run (one stream each), its launches
+
+template <class T>
+void record(const char* what, const T* v, int32_t n)
+{
+    if (g_runs.empty()) g_runs.emplace_back();
+    g_runs.back().append(what).append(reinterpret_cast<const char*>(v), (size_t)n * sizeof(T));
+}
 
 SwArgs one_task(const SwArgs& a, const SwTask* t, int32_t* ticket)
 {
@@ -71,21 +82,30 @@ const char* unit_fault(const SwArgs& a, const SwUnit* units, int32_t t, int32_t 
 
 namespace cm {
 
+cudaError_t launch_gather_stream(const uint8_t* db, const int64_t* off, const int32_t* ids, int32_t nb,
+                                 const int64_t* srow, uint8_t* stream, cudaStream_t st)
+{
+    g_runs.emplace_back();
+    return gather_stream(db, off, ids, nb, srow, stream, st);
+}
+
 cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaStream_t st)
 {
+    record("tile", a.tasks, a.ntasks);
     if (mode != kModePair && mode != kModeSeg16) return cudaErrorInvalidValue;
     return tile_launch(R, W, mode, grid, a, st);
 }
 
 cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaStream_t st)
 {
+    record("pairs", a.tasks, a.ntasks);
     if (grid < 1 || W != 16) return cudaErrorInvalidValue;
     if (*a.task_counter != 0) { contract_error(a, "task ticket not zeroed"); return cudaSuccess; }
     for (int32_t i = 0; i < a.ntasks; ++i) {
         const SwTask& t = a.tasks[i];
         if (sw16_pair_smem(t.R, t.mode) > smem) { contract_error(a, "profile too large"); return cudaSuccess; }
         int32_t ticket;
-        const cudaError_t e = launch_sw16(t.R, W, t.mode, grid, one_task(a, &t, &ticket), st);
+        const cudaError_t e = tile_launch(t.R, W, t.mode, grid, one_task(a, &t, &ticket), st);
         if (e != cudaSuccess) return e;
     }
     *a.task_counter = a.ntasks;
@@ -96,6 +116,7 @@ cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_
 {
     if (grid < 1 || warps < 1 || warps > kSingleWarps) return cudaErrorInvalidValue;
     const int32_t n = a.ranges[a.nranges];
+    record("single", a.units, n);
     if (a.nranges < 1 || a.nranges > grid || a.ranges[0] != 0) { contract_error(a, "ranges"); return cudaSuccess; }
     std::vector<int32_t> range_of((size_t)n, 0);
     std::vector<char> home((size_t)a.nranges, 0);
@@ -136,4 +157,27 @@ cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_
 
 }  // namespace cm
 
-int main() { return api_mock_main(); }
+// The autotuner on a set of the lengths of argv: every plan it makes runs twice, and both runs have
+// to launch the same work in the same order.
+int main(int argc, char** argv)
+{
+    if (argc < 2) return api_mock_main();
+    cm_ctx* ctx = nullptr;
+    if (cm_create(&ctx, 0)) return 1;
+    g_sym = true;
+    g_off.assign(1, 0);
+    for (int i = 1; i < argc; ++i) g_off.push_back(g_off.back() + std::atoll(argv[i]));
+    std::vector<uint8_t> seqs((size_t)g_off.back(), 3);
+    std::vector<int8_t> mat(400, 1);
+    int32_t w = 0, rows = 0;
+    const int r = cm_autotune(ctx, seqs.data(), g_off.data(), argc - 1, mat.data(), 11, 1, 0, nullptr, &w,
+                              &rows, 0);
+    cm_stats st{};
+    cm_get_stats(ctx, &st);
+    int differ = 0;
+    for (size_t i = 0; i + 1 < g_runs.size(); i += 2) differ += g_runs[i] != g_runs[i + 1];
+    std::printf("error %d runs %zu differ %d cells %lld of %lld\n", r, g_runs.size(), differ,
+                (long long)g_cells_done, (long long)st.cells);
+    cm_destroy(ctx);
+    return 0;
+}

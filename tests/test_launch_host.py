@@ -60,3 +60,15 @@ def test_pipelined_tasks_stay_in_one_range(exe):
         H.add("score 0 %d %s" % (len(pairs), flat),
               api._expect_values("score", [api._score(a, b, L, False) for a, b in pairs]))
     H.run()
+
+
+@pytest.mark.parametrize("lengths", [[300] * 12 + [700] * 9,              # no query pair at 16 warps
+                                     list(range(520, 920, 5))])            # a merged launch
+def test_autotune_times_the_work_it_counts(exe, lengths):
+    """The autotuner runs a plan to warm up and again for the time: both runs launch the same tasks
+    and units in the same order, and all of the cells that it divides by the time."""
+    out = subprocess.run([exe] + [str(n) for n in lengths], capture_output=True, text=True)
+    assert "contract violated" not in out.stderr, out.stderr
+    words = out.stdout.split()
+    assert words[:6] == ["error", "0", "runs", "24", "differ", "0"], out.stdout
+    assert words[7] == words[9], out.stdout
