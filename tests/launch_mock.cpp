@@ -9,13 +9,18 @@
 
 #define launch_sw16 tile_launch
 #define launch_gather_stream gather_stream
+#define launch_long_cells long_cells
 #define main api_mock_main
 #include "api_mock.cpp"
 #undef main
+#undef launch_long_cells
 #undef launch_gather_stream
 #undef launch_sw16
 
 namespace {
+
+cm_ctx* g_ctx = nullptr;                           // for the size of its boundary buffer
+int g_huge = 0;                                    // launches of the kernel of scores from 2^28
 
 std::vector<std::string> g_runs;                   // per plan run (one stream each), its launches
 
@@ -96,6 +101,21 @@ cudaError_t launch_sw16(int R, int W, int mode, int grid, const SwArgs& a, cudaS
     return tile_launch(R, W, mode, grid, a, st);
 }
 
+// without units: the kernel of huge scores, with its slots behind the strips' boundary columns
+cudaError_t launch_long_cells(int grid, const SwArgs& a, const CellJob* jobs, int32_t n, int32_t* counter,
+                              int32_t* res, cudaStream_t st)
+{
+    if (!a.cell_units) {
+        ++g_huge;
+        const DevBuf& b = g_ctx->buf[B_BND];
+        const int64_t end = (a.bnd - static_cast<uint2*>(b.p)) + (int64_t)grid * kLongSlots * a.bnd_stride;
+        if (a.bnd < b.p || end * (int64_t)sizeof(uint2) > (int64_t)b.cap) contract_error(a, "slots outside the buffer");
+        for (int32_t i = 0; i < n; ++i)
+            if (jobs[i].m > a.bnd_stride) contract_error(a, "rows beyond a slot");
+    }
+    return long_cells(grid, a, jobs, n, counter, res, st);
+}
+
 cudaError_t launch_sw16_pairs(int W, int grid, int smem, const SwArgs& a, cudaStream_t st)
 {
     record("pairs", a.tasks, a.ntasks);
@@ -157,27 +177,44 @@ cudaError_t launch_sw16_single(int grid, int warps, const SwArgs& a, cudaStream_
 
 }  // namespace cm
 
-// The autotuner on a set of the lengths of argv: every plan it makes runs twice, and both runs have
-// to launch the same work in the same order.
+// "cells": the cells of every ordered pair of a set of the given lengths, with a matrix of 127: as
+// the fake similarity gives them, and how many launches went to the kernel of huge scores.
+// "autotune": the autotuner on such a set; every plan it makes runs twice, and both runs have to
+// launch the same work in the same order.
 int main(int argc, char** argv)
 {
-    if (argc < 2) return api_mock_main();
-    cm_ctx* ctx = nullptr;
-    if (cm_create(&ctx, 0)) return 1;
+    if (argc < 3) return api_mock_main();
+    if (cm_create(&g_ctx, 0)) return 1;
     g_sym = true;
     g_off.assign(1, 0);
-    for (int i = 1; i < argc; ++i) g_off.push_back(g_off.back() + std::atoll(argv[i]));
+    for (int i = 2; i < argc; ++i) g_off.push_back(g_off.back() + std::atoll(argv[i]));
+    const int32_t n = argc - 2;
     std::vector<uint8_t> seqs((size_t)g_off.back(), 3);
-    std::vector<int8_t> mat(400, 1);
-    int32_t w = 0, rows = 0;
-    const int r = cm_autotune(ctx, seqs.data(), g_off.data(), argc - 1, mat.data(), 11, 1, 0, nullptr, &w,
-                              &rows, 0);
-    cm_stats st{};
-    cm_get_stats(ctx, &st);
-    int differ = 0;
-    for (size_t i = 0; i + 1 < g_runs.size(); i += 2) differ += g_runs[i] != g_runs[i + 1];
-    std::printf("error %d runs %zu differ %d cells %lld of %lld\n", r, g_runs.size(), differ,
-                (long long)g_cells_done, (long long)st.cells);
-    cm_destroy(ctx);
+    std::vector<int8_t> mat(400, 127);
+    if (std::strcmp(argv[1], "cells") == 0) {
+        std::vector<int32_t> p, got((size_t)n * n * 5);
+        for (int32_t x = 0; x < n; ++x)
+            for (int32_t y = 0; y < n; ++y) p.insert(p.end(), {x, y});
+        const int r = sw_cells_batch(g_ctx, seqs.data(), g_off.data(), n, p.data(), (int64_t)n * n, mat.data(),
+                                     11, 1, got.data(), 0);
+        int differ = 0;
+        for (int32_t q = 0; q < n * n; ++q) {
+            int64_t c[5];
+            fake_cells(p[2 * q], p[2 * q + 1], c);
+            for (int k = 0; k < 5; ++k) differ += c[k] != got[5 * (size_t)q + k];
+        }
+        std::printf("error %d differ %d huge %d\n", r, differ, g_huge);
+    } else {
+        int32_t w = 0, rows = 0;
+        const int r = cm_autotune(g_ctx, seqs.data(), g_off.data(), n, mat.data(), 11, 1, 0, nullptr, &w,
+                                  &rows, 0);
+        cm_stats st{};
+        cm_get_stats(g_ctx, &st);
+        int differ = 0;
+        for (size_t i = 0; i + 1 < g_runs.size(); i += 2) differ += g_runs[i] != g_runs[i + 1];
+        std::printf("error %d runs %zu differ %d cells %lld of %lld\n", r, g_runs.size(), differ,
+                    (long long)g_cells_done, (long long)st.cells);
+    }
+    cm_destroy(g_ctx);
     return 0;
 }

@@ -67,8 +67,19 @@ def test_pipelined_tasks_stay_in_one_range(exe):
 def test_autotune_times_the_work_it_counts(exe, lengths):
     """The autotuner runs a plan to warm up and again for the time: both runs launch the same tasks
     and units in the same order, and all of the cells that it divides by the time."""
-    out = subprocess.run([exe] + [str(n) for n in lengths], capture_output=True, text=True)
+    out = subprocess.run([exe, "autotune"] + [str(n) for n in lengths], capture_output=True, text=True)
     assert "contract violated" not in out.stderr, out.stderr
     words = out.stdout.split()
     assert words[:6] == ["error", "0", "runs", "24", "differ", "0"], out.stdout
     assert words[7] == words[9], out.stdout
+
+
+@pytest.mark.parametrize("lengths,huge", [([2200000, 3000, 2300000, 200, 2500], True),
+                                          ([2100000, 2100000, 3000], False)])
+def test_cells_of_huge_scores_have_their_slots(exe, lengths, huge):
+    """Pairs that may score 2^28 take the long pairs of their round to the kernel for such scores,
+    whose slots lie behind the boundary columns of the other pairs' strips."""
+    out = subprocess.run([exe, "cells"] + [str(n) for n in lengths], capture_output=True, text=True)
+    assert "contract violated" not in out.stderr, out.stderr
+    words = out.stdout.split()
+    assert words[:4] == ["error", "0", "differ", "0"] and (int(words[5]) > 0) == huge, out.stdout
