@@ -97,12 +97,14 @@ int cm_set_tuning(cm_ctx *ctx, int32_t warps_per_cta, int32_t rows_per_warp);
  * 0 restores the default of 2^32. */
 int cm_set_batch_limit(cm_ctx *ctx, int64_t max_slots);
 
-/* Bound on the one device wait of the library: a pass of the whole-CTA long-pair kernels
- * (int32 rescoring and alignment cells of pairs of >= 2,048 x 512 residues) waits for the
- * rows its predecessor pass has written.  Such a wait always ends in a correct run; after
- * `polls` polls of ~100 ns each it gives up instead, the call returns CM_ERR_TIMEOUT with
- * nothing written, and the context stays usable.  0 restores the default of 2^24 polls
- * (~1.7 s).  A small value exists to exercise that error path. */
+/* Bound on the device waits of the int32 passes over long pairs (rescoring and alignment cells of
+ * pairs of >= 2,048 x 512 residues): the warp of a column strip waits for the rows that the strip
+ * before it has written.  Such a wait always ends in a correct run; after `polls` polls of ~100 ns
+ * each it gives up instead, the call returns CM_ERR_TIMEOUT with nothing written, and the context
+ * stays usable.  0 restores the default of 2^24 polls (~1.7 s).  A small value exists to exercise
+ * that error path.  The other kernels whose warps wait for one another's column passes (strips of
+ * shorter pairs, lone queries of more than 512 residues, tracebacks) wait the same way, always with
+ * the bound of 2^24 polls. */
 int cm_set_wait_limit(cm_ctx *ctx, int32_t polls);
 
 /* Autotuner: scores the all-against-all of a length-stratified sample of `sample_seqs` of the

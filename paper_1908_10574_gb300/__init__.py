@@ -152,8 +152,8 @@ class Context:
         _L.check(self._h, _L.lib().cm_set_batch_limit(self._h, int(max_slots)))
 
     def set_wait_limit(self, polls=0):
-        """Polls (~100 ns each) before the long-pair pipeline wait gives up with
-        CM_ERR_TIMEOUT (0: the default of 2^24)."""
+        """Polls (~100 ns each) before a wait of the int32 passes over long pairs gives up with
+        CM_ERR_TIMEOUT (0: the default of 2^24, which bounds every other kernel's waits)."""
         _L.check(self._h, _L.lib().cm_set_wait_limit(self._h, int(polls)))
 
     # ---- entry points ---------------------------------------------------------------------
