@@ -21,7 +21,9 @@
 // is taken by another warp and trails the one before it by 32 row groups (progress.cuh), so a
 // long pair is a pipeline; the warp of the last pass walks back.  Pairs run in rounds whose
 // scratch (direction words, boundary column, runs) fits a budget.
-// Bound: about 15 instructions per cell.  Measured on one GB300, 2,000 pairs of up to 1,500
+// Bound: issue and the ALU pipe (54 and 65 % busy on an active SM), with 12 warps of 167 registers;
+// some 15 instructions update a cell, 45 are issued for it with the wavefront's fill, the padding of
+// short spans, the profiles and the walks.  Measured on one GB300, 2,000 pairs of up to 1,500
 // residues (4.6e8 cells): 295 ms with one thread per pair and a byte per cell, 4.9 ms with one
 // warp per pair (the longest pairs crowd a few SMs), 1.5 ms with a warp per pass.
 #include <algorithm>

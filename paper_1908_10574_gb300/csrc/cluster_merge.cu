@@ -813,7 +813,7 @@ int Driver::finish(std::vector<int32_t>& final_set, cm_result* res)
     // intra-cluster all-against-all: one TRI block per cluster (members in length order).  A
     // cluster with two or more members longer than kLongSubject splits: TRI over its short
     // members, a CROSS block of the long members (queries) against the short ones, and the
-    // long x long pairs straight on the int32 whole-CTA kernels (in a TRI block each of them
+    // long x long pairs straight on the int32 strips (in a TRI block each of them
     // is one warp's stream over dozens of column passes while the CTA's other warps wait,
     // and such pairs of one family exceed the int16 range and are rescored anyway).
     std::vector<int32_t> ids, ll;

@@ -4,13 +4,13 @@
 //
 // conv_tc_kernel<CIN, NOUT, EPI>: out[r, n] = sum_t sum_c X[r + t - 4, c] * Wk[n, t*CIN + c]
 //   (forward: Wk[n, t*CIN + c] = W[t][c][n]; backward-data: X = dY, Wk[c, t*128 + n] =
-//   W[8-t][c][n]).  A tile is 128 rows x NOUT channels: K runs over the 9 taps x CIN channels
-//   in stages of BK channels; a stage's A tile is the 128 rows starting at r0 + t - 4, loaded
-//   by TMA straight from the activation matrix (rows before 0 or past the end come back as
-//   zeros), and its B tile the matching BK columns of Wk.  Persistent: one CTA per SM walks
-//   the tiles; one thread streams the stages of every tile through a deep mbarrier ring,
-//   one thread issues the MMAs of a tile into one of two TMEM accumulators, and four warps
-//   read the other accumulator back and apply the epilogue meanwhile (details below).
+//   W[8-t][c][n]).  A tile is 128 rows x NOUT channels: K runs over the 9 taps x CIN channels, a
+//   stage to a tap.  The tile's rows r0 - 4 .. r0 + 131 are loaded once by TMA straight from the
+//   activation matrix (rows before 0 or past the end come back as zeros) and tap t reads them
+//   from row t on; a stage holds the tap's CIN columns of Wk.  Persistent: one CTA per SM walks
+//   the tiles; one thread streams rows and stages through mbarrier rings, one warp issues the
+//   MMAs of a tile into one of two TMEM accumulators, and eight or sixteen warps read the other
+//   accumulator back and apply the epilogue meanwhile (details below).
 // wgrad_tc_kernel<CIN>: part[chunk][m = t*CIN + c][n] = sum over the chunk's rows r of
 //   X[r + t - 4, c] * dY[r, n] -- a GEMM whose K runs over rows.  Both operands are read
 //   MN-major (channels contiguous, one row per K index), so the tap shift stays on the row

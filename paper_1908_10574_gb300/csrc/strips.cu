@@ -11,7 +11,7 @@
 // the last strip writes the job's result.
 // Bound: the ALU pipe, 3.5 half-rate DPX operations per cell and the dot product's share.
 // Measured on one GB300, 20,000 pairs of related proteins (1.0e10 cells in both directions):
-// 5.4 ms (1.9 Tcells/s, the ALU pipe 74 % busy); 14.4 ms for a warp per job with an int32
+// 5.4 ms (1.9 Tcells/s, the ALU pipe 73 % busy); 14.4 ms for a warp per job with an int32
 // profile (38 KB: five warps on an SM) and four more operations per cell to track the position,
 // plus whole CTAs for the long jobs.  Two rows per step instead of four: the same time (less
 // wavefront to fill, more overhead per row).  Rescoring of 24 pairs of 8,000-12,000 residues

@@ -28,8 +28,9 @@
 // Bound: the ALU pipe, 5.5 of its half-rate operations per packed column (E, F, D, H, half a
 // running maximum and the permute).  Measured on one GB300 against CTAs of 16 warps per query
 // and a launch per tile: 50,000 pairs of 5,000 proteins (ten subjects per query) 26.6 -> 9.4 ms
-// per call (6.5 with the pairs ordered by a counting sort), the kernel 20+ -> 4.9 ms at 59 % ALU; one query against 200 proteins 0.84 -> 0.37 ms;
-// 24 pairs of 8,000-12,000 residues 84.5 -> 13.0 ms (9.8 ms of it the int32 rescoring).  The cell
+// per call (6.4 with the pairs ordered by a counting sort), the kernel 20+ -> 4.2 ms (ALU pipe 63 %
+// busy on an active SM, SMs active 77 % of the launch); one query against 200 proteins 0.84 -> 0.4 ms;
+// 24 pairs of 8,000-12,000 residues 84.5 -> 5.9 ms (3.5 ms here, 2.2 the int32 rescoring).  The cell
 // update of sw16_kernel.cuh with the floor in F (profile bytes of S + o, D a plain add) was 2 %
 // slower here: twelve warps wait for latency before the ALU pipe is full.
 #include "progress.cuh"
